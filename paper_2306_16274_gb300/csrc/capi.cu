@@ -198,8 +198,10 @@ lbm::Bufs bufs(const lbm_ctx* c) {
 cudaError_t run_psi(lbm_ctx* c) {
     if (!c->kp.multiphase && !c->f16) return cudaSuccess;
     const int s = has_solids(c);
-    return c->Q == 19 ? lbm::launch_psi_q19(c->kp, c->parity, s, bufs(c), c->stream)
-                      : lbm::launch_psi_q27(c->kp, c->parity, s, bufs(c), c->stream);
+    lbm::KParams k = c->kp;
+    k.down = 1;   // against the collide pass's direction
+    return c->Q == 19 ? lbm::launch_psi_q19(k, c->parity, s, bufs(c), c->stream)
+                      : lbm::launch_psi_q27(k, c->parity, s, bufs(c), c->stream);
 }
 
 // Tensor map of one population copy for the staged one-pass kernel: a 4-D array (x, y, z,
@@ -253,8 +255,10 @@ cudaError_t run_onepass(lbm_ctx* c) {
         e = c->Q == 19 ? lbm::launch_onepass_tma_q19(c->kp, c->tmap[k], c->status, extra, cycles, c->stream)
                        : lbm::launch_onepass_tma_q27(c->kp, c->tmap[k], c->status, extra, cycles, c->stream);
     } else {
-        e = c->Q == 19 ? lbm::launch_onepass_q19(c->kp, c->status, c->stream)
-                       : lbm::launch_onepass_q27(c->kp, c->status, c->stream);
+        lbm::KParams k = c->kp;
+        k.down = (int)(c->t & 1);   // against the step before
+        e = c->Q == 19 ? lbm::launch_onepass_q19(k, c->status, c->stream)
+                       : lbm::launch_onepass_q27(k, c->status, c->stream);
     }
     std::swap(c->f, c->f2);
     for (int i = 0; i < 27; ++i) std::swap(c->kp.fq[i], c->kp.gq[i]);
@@ -274,9 +278,10 @@ cudaError_t launch_collide(const lbm_ctx* c, const lbm::KParams& k, int solids) 
 
 cudaError_t run_collide(lbm_ctx* c) {
     cudaError_t e;
+    lbm::KParams k = c->kp;
+    k.down = !k.multiphase && !c->f16 ? c->parity : 0;   // without a density pass: against the step before
     if (zwalls_only(c)) {
         // each slot is read and written by one cell only, so the three plane ranges are independent
-        lbm::KParams k = c->kp;
         k.zlo = 1;
         k.zhi = k.nz - 1;
         e = launch_collide(c, k, 0);
@@ -287,7 +292,7 @@ cudaError_t run_collide(lbm_ctx* c) {
         k.zhi = k.nz;
         if (e == cudaSuccess) e = launch_collide(c, k, 1);
     } else {
-        e = launch_collide(c, c->kp, has_solids(c));
+        e = launch_collide(c, k, has_solids(c));
     }
     if (c->f16) c->rs ^= 1;   // the slots are now relative to the densities the collide pass used
     return e;

@@ -43,6 +43,7 @@ struct KParams {
     float* fq[27];                // base of population plane i (f + i * plane); cells < 2^31
     int zchunk;                   // z planes per collide block (0 = automatic)
     int zlo, zhi;                 // planes [zlo, zhi) the whole-grid collide kernels march through
+    int down;                     // 1: the launch takes the planes from the top down
     float* gq[27];                // one-pass layout: planes of the copy the step writes
     // shifted FP16 store in the x-paired layout (even nx, x periodic, no solid mask): word w of a
     // row holds cells w (low half) and w + hx (high half), hx = nx / 2, so a shift by one cell in
