@@ -255,10 +255,8 @@ cudaError_t run_onepass(lbm_ctx* c) {
         e = c->Q == 19 ? lbm::launch_onepass_tma_q19(c->kp, c->tmap[k], c->status, extra, cycles, c->stream)
                        : lbm::launch_onepass_tma_q27(c->kp, c->tmap[k], c->status, extra, cycles, c->stream);
     } else {
-        lbm::KParams k = c->kp;
-        k.down = (int)(c->t & 1);   // against the step before
-        e = c->Q == 19 ? lbm::launch_onepass_q19(k, c->status, c->stream)
-                       : lbm::launch_onepass_q27(k, c->status, c->stream);
+        e = c->Q == 19 ? lbm::launch_onepass_q19(c->kp, c->status, c->stream)
+                       : lbm::launch_onepass_q27(c->kp, c->status, c->stream);
     }
     std::swap(c->f, c->f2);
     for (int i = 0; i < 27; ++i) std::swap(c->kp.fq[i], c->kp.gq[i]);

@@ -73,10 +73,10 @@ __device__ __forceinline__ void psi_column(const KParams& kp, const GM& g, const
 
 // Consecutive passes sweep the planes in opposite directions (KParams::down), so that a pass starts on the
 // planes that the one before it left in the L2 cache: collide upwards, density downwards; single-phase
-// (in-place or one-pass) steps turn round after every step.  What is found there is about 50 MB a pass
+// steps turn round after every step.  What is found there is about 50 MB a pass
 // however large the domain is.  us a step, always upwards / turning: D3Q19 128^3 90.1 / 82.6, 160^3 165.8 /
 // 160.4, 256^3 624 / 618, single-phase 128^3 53.4 / 47.0; D3Q27 128^3 122.9 / 115.2, 256^3 867 / 860.
-// (96^3 fits the L2 either way: 35.8 / 35.8.)
+// (96^3 fits the L2 either way: 35.8 / 35.8.)  The one-pass kernel does not turn: 7 % slower on D3Q27 192^3.
 __device__ __forceinline__ int swept_block(int down) {
     return down ? (int)gridDim.z - 1 - (int)blockIdx.z : (int)blockIdx.z;
 }
@@ -730,7 +730,7 @@ __global__ void __launch_bounds__(32 * BY, MINB) collide_onepass_kernel(const KP
     static_assert(HALO <= 32 * BY, "one border cell per thread at most");
     __shared__ float ring[4][RP];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + 32 * ty;
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * BY, z0 = swept_block(kp.down) * zchunk;
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * BY, z0 = blockIdx.z * zchunk;
     const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
     const int x = x0 + tx, y = y0 + ty;
     const bool act = x < nx && y < ny;
