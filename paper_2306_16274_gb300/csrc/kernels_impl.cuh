@@ -71,6 +71,18 @@ __device__ __forceinline__ void psi_column(const KParams& kp, const GM& g, const
     }
 }
 
+// Step kernels of one stream overlap at their ends: a kernel waits here for the previous one to have
+// finished (its memory visible) before it reads or writes anything, and then lets the next one fill the SMs
+// as soon as all its own blocks have come this far.  Every block of every step kernel waits, so a kernel that
+// has finished implies that all before it have, and at most two are on the SMs.  Saves the launch and the first
+// fetch of the parameters, about 2 us a kernel: us a step without / with, D3Q19 32^3 10.3 / 6.0, 64^3 17.4 /
+// 13.3, 96^3 35.7 / 31.8, 128^3 82.0 / 78.2, 200 x 200 x 100 with z walls (four kernels) 182.5 / 174.6,
+// 256^3 619.0 / 615.3; D3Q27 61 x 83 x 70 28.0 / 24.0.
+__device__ __forceinline__ void dep_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Consecutive passes sweep the planes in opposite directions (KParams::down), so that a pass starts on the
 // planes that the one before it left in the L2 cache: collide upwards, density downwards; single-phase
 // steps turn round after every step.  What is found there is about 50 MB a pass
@@ -89,6 +101,7 @@ __global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_kernel(KParams kp, float*
     const KGeom g{kp};
     const PlanePtrsT<typename std::conditional<F16, __half, float>::type> addr{kp};
     const int z = swept_block(kp.down);
+    dep_wait();
     psi_column<PARITY, SOLIDS, F16>(kp, g, addr, psi, nbmask, status, blockIdx.x * PSI_BX + threadIdx.x,
                                     blockIdx.y * PSI_BY + threadIdx.y, z, z + 1, rsrc, rdst);
 }
@@ -190,7 +203,7 @@ __device__ __forceinline__ void load_psi_plane(float* slot, const float* __restr
 #pragma unroll
     for (int s = 0; s < TS::SLOTS; ++s) {
         const int k = tid + s * TS::NT;
-        if (k < TS::RP) slot[k] = (zok && gok[s]) ? __ldg(psi + bounded(zb + goff[s], (unsigned long long)nxy * nz)) : 0.0f;
+        if (k < TS::RP) slot[k] = (zok && gok[s]) ? ldnow(psi + bounded(zb + goff[s], (unsigned long long)nxy * nz)) : 0.0f;
     }
 }
 
@@ -206,7 +219,7 @@ __device__ __forceinline__ void fetch_psi_plane(float (&v)[TS::SLOTS], const flo
 #pragma unroll
     for (int s = 0; s < TS::SLOTS; ++s) {
         const int k = tid + s * TS::NT;
-        v[s] = (k < TS::RP && zok && gok[s]) ? __ldg(psi + bounded(zb + goff[s], (unsigned long long)nxy * nz)) : 0.0f;
+        v[s] = (k < TS::RP && zok && gok[s]) ? ldnow(psi + bounded(zb + goff[s], (unsigned long long)nxy * nz)) : 0.0f;
     }
 }
 template <class TS>
@@ -340,7 +353,7 @@ __device__ __forceinline__ void collide_tile(const KParams& kp, const GM& g, con
         float rho, ux, uy, uz;
         collide<Q>(kp, p, Fo, rho, ux, uy, uz);
         if (!(rho > 0.0f) || !(fabsf(ux) + fabsf(uy) + fabsf(uz) < 1e30f)) atomicOr(status, ST_UNSTABLE);
-        if (F16) normalize<Q>(p, __ldg(rown + o.c));
+        if (F16) normalize<Q>(p, ldnow(rown + o.c));
         store32<Q, PARITY, SOLIDS>(addr, o, bits, p);
     }
 }
@@ -354,6 +367,7 @@ __global__ void __launch_bounds__(ZmTile::NT, ZM_MINB) collide_kernel(const KPar
     __shared__ float ring[F16 ? 8 : 4][ZmTile::RP];
     const KGeom g{kp};
     const PlanePtrsT<typename std::conditional<F16, __half, float>::type> addr{kp};
+    dep_wait();
     collide_tile<ZmTile, PARITY, SOLIDS, MULTIPHASE, F16, true>(kp, g, addr, psi, nbmask, status, blockIdx.x * ZM_BX,
                                                         blockIdx.y * ZM_BY, kp.zlo + swept_block(kp.down) * zchunk,
                                                         zchunk, kp.zhi, ring, ring + 4, rsrc, rown);
@@ -413,10 +427,12 @@ __device__ __forceinline__ float half_hi(uint32_t v) { return __half2float(__ush
 __device__ __forceinline__ uint32_t ldword(const uint32_t* p) {
 #if LBM_LDWORD_HINT == 2
     uint32_t v;
-    asm("ld.global.nc.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 #else
-    return __ldg(p);
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
 #endif
 }
 __device__ __forceinline__ void stword(uint32_t* p, uint32_t v) {
@@ -507,8 +523,8 @@ __device__ __forceinline__ void fetch_pair_plane(float2 (&v)[PR_SLOTS], const fl
     for (int s = 0; s < PR_SLOTS; ++s) {
         const int k = tid + s * PR_NT;
         if (k < PR_RP && zok && g.ok[s]) {
-            const float a = __ldg(fld + bounded(zb + g.off[s], (unsigned long long)nxy * nz));
-            const float b = __ldg(fld + bounded(zb + g.off[s] + hx, (unsigned long long)nxy * nz));
+            const float a = ldnow(fld + bounded(zb + g.off[s], (unsigned long long)nxy * nz));
+            const float b = ldnow(fld + bounded(zb + g.off[s] + hx, (unsigned long long)nxy * nz));
             v[s] = g.sw[s] ? make_float2(b, a) : make_float2(a, b);
         } else {
             v[s] = make_float2(0.0f, 0.0f);
@@ -556,6 +572,7 @@ __global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_pair_kernel(KParams kp, f
                                                                  float* __restrict__ rdst) {
     const int hx = kp.hx, nx = kp.nx, ny = kp.ny, nz = kp.nz;
     const int w = blockIdx.x * PSI_BX + threadIdx.x, y = blockIdx.y * PSI_BY + threadIdx.y, z = swept_block(kp.down);
+    dep_wait();
     if (w >= hx || y >= ny) return;
     const uint32_t nxy = (uint32_t)nx * (uint32_t)ny;
     WOff o;
@@ -616,6 +633,7 @@ __global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const KPar
     const uint32_t selL = w == 0 ? PERM_SWAP : PERM_KEEP, selR = w == hx - 1 ? PERM_SWAP : PERM_KEEP;
     const uint32_t rowA = (uint32_t)(y < ny ? y : 0) * (uint32_t)nx + (uint32_t)(w < hx ? w : 0);   // low cell in its plane
 
+    dep_wait();
     // words and own densities of the first plane, then of plane z+1 while plane z is computed
     uint32_t wn[Q];
     float rn[2] = {0.0f, 0.0f};
@@ -624,8 +642,8 @@ __global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const KPar
         set_wplane(o, z0, nz, wpl);
         bits_n = SOLIDS ? solid_bits32<Q>(g, nullptr, 0u, w, y, z0) : 0u;
         gather_pair<PARITY, SOLIDS>(addr, o, bits_n, selL, selR, wn);
-        rn[0] = __ldg(rown + (uint32_t)z0 * nxy + rowA);
-        rn[1] = __ldg(rown + (uint32_t)z0 * nxy + rowA + hx);
+        rn[0] = ldnow(rown + (uint32_t)z0 * nxy + rowA);
+        rn[1] = ldnow(rown + (uint32_t)z0 * nxy + rowA + hx);
     }
     float2 pv[PR_SLOTS], rv[PR_SLOTS];
     if (MULTIPHASE) fetch_pair_plane(pv, psi, z0 + 1, nz, g.wall_z(), nxy, hx, src, tid);
@@ -658,8 +676,8 @@ __global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const KPar
             set_wplane(o, z, nz, wpl);
             bits_n = SOLIDS ? solid_bits32<Q>(g, nullptr, 0u, w, y, z) : 0u;
             gather_pair<PARITY, SOLIDS>(addr, o, bits_n, selL, selR, wn);
-            rn[0] = __ldg(rown + (uint32_t)z * nxy + rowA);
-            rn[1] = __ldg(rown + (uint32_t)z * nxy + rowA + hx);
+            rn[0] = ldnow(rown + (uint32_t)z * nxy + rowA);
+            rn[1] = ldnow(rown + (uint32_t)z * nxy + rowA + hx);
         }
 #pragma unroll
         for (int i = 0; i < Q; ++i) wv[i] = wn[i];
@@ -669,8 +687,8 @@ __global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const KPar
             set_wplane(o, z + 1, nz, wpl);
             bits_n = SOLIDS ? solid_bits32<Q>(g, nullptr, 0u, w, y, z + 1) : 0u;
             gather_pair<PARITY, SOLIDS>(addr, o, bits_n, selL, selR, wn);
-            rn[0] = __ldg(rown + (uint32_t)(z + 1) * nxy + rowA);
-            rn[1] = __ldg(rown + (uint32_t)(z + 1) * nxy + rowA + hx);
+            rn[0] = ldnow(rown + (uint32_t)(z + 1) * nxy + rowA);
+            rn[1] = ldnow(rown + (uint32_t)(z + 1) * nxy + rowA + hx);
         }
         set_wplane(o, z, nz, wpl);
         // wv ends up holding the outputs: the low cell's packed results replace the low halves it
@@ -783,6 +801,7 @@ __global__ void __launch_bounds__(32 * BY, MINB) collide_onepass_kernel(const KP
     };
 
     float pn[Q];
+    dep_wait();
     if (MULTIPHASE) {
         float tmp[Q];
         plane_psi(ring[0], z0 - 1, tmp);
@@ -1344,6 +1363,22 @@ dim3 cs_grid(const KParams& kp) {
     return dim3((kp.nx + CS_BX - 1) / CS_BX, (kp.ny + CS_BY - 1) / CS_BY, (kp.nz + CS_BZ - 1) / CS_BZ);
 }
 
+// Launch of a step kernel, whose blocks may start before the previous kernel of the stream has finished and
+// wait for it in dep_wait().
+template <class... KA, class... A>
+cudaError_t launch_dep(void (*kernel)(KA...), dim3 g, dim3 b, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g;
+    cfg.blockDim = b;
+    cfg.stream = st;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KA(args)...);
+}
+
 // Launches one collide_kernel instantiation (internal linkage: each lattice's translation unit
 // must launch its own kernels).  LBM_ZM_CARVEOUT >= 0 sets the preferred shared-memory carveout
 // (percent) once; the default leaves the driver's choice, which keeps L1 large for the
@@ -1362,8 +1397,7 @@ cudaError_t launch_collide_variant(dim3 g, dim3 b, cudaStream_t st, const KParam
             configured = true;
         }
     }
-    collide_kernel<PARITY, SOLIDS, MULTIPHASE, F16><<<g, b, 0, st>>>(kp, B.psi, B.nbmask, B.status, zc, B.rsrc, B.rnew);
-    return cudaGetLastError();
+    return launch_dep(collide_kernel<PARITY, SOLIDS, MULTIPHASE, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, zc, B.rsrc, B.rnew);
 }
 
 template <bool F16>
@@ -1381,12 +1415,12 @@ cudaError_t launch_collide_store(dim3 g, dim3 b, cudaStream_t st, const KParams&
 }
 
 template <bool F16>
-void launch_psi_store(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, int parity, int solids, const Bufs& B) {
-    if (parity == 2) psi_kernel<2, false, F16><<<g, b, 0, st>>>(kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    else if (parity == 0 && !solids) psi_kernel<0, false, F16><<<g, b, 0, st>>>(kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    else if (parity == 0) psi_kernel<0, true, F16><<<g, b, 0, st>>>(kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    else if (!solids) psi_kernel<1, false, F16><<<g, b, 0, st>>>(kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    else psi_kernel<1, true, F16><<<g, b, 0, st>>>(kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
+cudaError_t launch_psi_store(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, int parity, int solids, const Bufs& B) {
+    if (parity == 2) return launch_dep(psi_kernel<2, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
+    if (parity == 0 && !solids) return launch_dep(psi_kernel<0, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
+    if (parity == 0) return launch_dep(psi_kernel<0, true, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
+    if (!solids) return launch_dep(psi_kernel<1, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
+    return launch_dep(psi_kernel<1, true, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
 }
 
 template <bool F16>
@@ -1451,16 +1485,14 @@ cudaError_t launch_psi_batch_shape(const KParams& phys, const BatchDomTable& dom
 cudaError_t LBM_CAT(launch_psi_q, LBM_Q)(const KParams& kp, int parity, int solids, const Bufs& B, cudaStream_t st) {
     if (B.paired) {
         const dim3 g((kp.hx + PSI_BX - 1) / PSI_BX, (kp.ny + PSI_BY - 1) / PSI_BY, kp.nz), b(PSI_BX, PSI_BY);
-        if (parity == 0 && !solids) psi_pair_kernel<0, false><<<g, b, 0, st>>>(kp, B.psi, B.status, B.rsrc, B.rnew);
-        else if (parity == 0) psi_pair_kernel<0, true><<<g, b, 0, st>>>(kp, B.psi, B.status, B.rsrc, B.rnew);
-        else if (!solids) psi_pair_kernel<1, false><<<g, b, 0, st>>>(kp, B.psi, B.status, B.rsrc, B.rnew);
-        else psi_pair_kernel<1, true><<<g, b, 0, st>>>(kp, B.psi, B.status, B.rsrc, B.rnew);
-        return cudaGetLastError();
+        if (parity == 0 && !solids) return launch_dep(psi_pair_kernel<0, false>, g, b, st, kp, B.psi, B.status, B.rsrc, B.rnew);
+        if (parity == 0) return launch_dep(psi_pair_kernel<0, true>, g, b, st, kp, B.psi, B.status, B.rsrc, B.rnew);
+        if (!solids) return launch_dep(psi_pair_kernel<1, false>, g, b, st, kp, B.psi, B.status, B.rsrc, B.rnew);
+        return launch_dep(psi_pair_kernel<1, true>, g, b, st, kp, B.psi, B.status, B.rsrc, B.rnew);
     }
     const dim3 g = psi_grid(kp), b(PSI_BX, PSI_BY);
-    if (B.f16) launch_psi_store<true>(g, b, st, kp, parity, solids, B);
-    else launch_psi_store<false>(g, b, st, kp, parity, solids, B);
-    return cudaGetLastError();
+    return B.f16 ? launch_psi_store<true>(g, b, st, kp, parity, solids, B)
+                 : launch_psi_store<false>(g, b, st, kp, parity, solids, B);
 }
 
 // z planes per block: enough blocks for a few waves of resident blocks on 152 SMs
@@ -1518,16 +1550,15 @@ cudaError_t LBM_CAT(launch_collide_q, LBM_Q)(const KParams& kp, int parity, int 
         const float* r0 = B.rsrc;
         const float* r1 = B.rnew;
         switch (key) {
-            case 0: collide_pair_kernel<0, false, false><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
-            case 1: collide_pair_kernel<0, false, true><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
-            case 2: collide_pair_kernel<0, true, false><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
-            case 3: collide_pair_kernel<0, true, true><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
-            case 4: collide_pair_kernel<1, false, false><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
-            case 5: collide_pair_kernel<1, false, true><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
-            case 6: collide_pair_kernel<1, true, false><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
-            default: collide_pair_kernel<1, true, true><<<g, b, 0, st>>>(kp, B.psi, B.status, zc, r0, r1); break;
+            case 0: return launch_dep(collide_pair_kernel<0, false, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+            case 1: return launch_dep(collide_pair_kernel<0, false, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+            case 2: return launch_dep(collide_pair_kernel<0, true, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+            case 3: return launch_dep(collide_pair_kernel<0, true, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+            case 4: return launch_dep(collide_pair_kernel<1, false, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+            case 5: return launch_dep(collide_pair_kernel<1, false, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+            case 6: return launch_dep(collide_pair_kernel<1, true, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+            default: return launch_dep(collide_pair_kernel<1, true, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
         }
-        return cudaGetLastError();
     }
     const int zc = collide_zchunk(kp);
     const int planes = kp.zhi - kp.zlo;
@@ -1621,9 +1652,8 @@ cudaError_t LBM_CAT(launch_onepass_q, LBM_Q)(const KParams& kp, unsigned* status
     // a chunk starts with two psi planes whose loads nothing overlaps
     const int zc = choose_zchunk(kp, 1.5, kp.nz, OP_BY, OP_MINB);
     const dim3 g((kp.nx + 31) / 32, (kp.ny + OP_BY - 1) / OP_BY, (kp.nz + zc - 1) / zc), b(32, OP_BY);
-    if (kp.multiphase) collide_onepass_kernel<true, OP_BY, OP_MINB><<<g, b, 0, st>>>(kp, status, zc);
-    else collide_onepass_kernel<false, OP_BY, OP_MINB><<<g, b, 0, st>>>(kp, status, zc);
-    return cudaGetLastError();
+    return kp.multiphase ? launch_dep(collide_onepass_kernel<true, OP_BY, OP_MINB>, g, b, st, kp, status, zc)
+                         : launch_dep(collide_onepass_kernel<false, OP_BY, OP_MINB>, g, b, st, kp, status, zc);
 }
 
 unsigned long long LBM_CAT(bounds_violations_q, LBM_Q)() {

@@ -97,30 +97,43 @@ __host__ __device__ constexpr float OMEGA(int i) {
 // 0.5946 / 0.2884 with plain read-only loads; evict-first stores 0.4209 (D3Q19) and 0.5999 ms (D3Q27)
 // against 0.4273 / 0.5946; loads bypassing L1 (.cg) no change; evict-first loads (.cs) 30 % slower.
 // Kept: prefetching loads on both lattices, evict-first stores on D3Q19.
+//
+// The step kernels load with ordinary (not read-only) loads in volatile assembly: a kernel may be resident
+// before the one that writes what it loads has finished, so the data are not read-only while it runs, and no
+// load may move above the wait for that one (dep_wait).  Read-only loads gave one-pass steps stale values.
 #ifndef LBM_LDPOP_HINT
 #define LBM_LDPOP_HINT 2
 #endif
 #ifndef LBM_STPOP_CS
 #define LBM_STPOP_CS (LBM_Q == 19)
 #endif
+__device__ __forceinline__ float ldnow(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ float ldpop(const float* p) {
 #if LBM_LDPOP_HINT == 1
     return __ldcg(p);
 #elif LBM_LDPOP_HINT == 2
     float v;
-    asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 #elif LBM_LDPOP_HINT == 3
     float v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 #elif LBM_LDPOP_HINT == 4
     return __ldcs(p);
 #else
-    return __ldg(p);
+    return ldnow(p);
 #endif
 }
-__device__ __forceinline__ float ldpop(const __half* p) { return __half2float(__ldg(p)); }
+__device__ __forceinline__ float ldpop(const __half* p) {
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __half2float(__ushort_as_half(v));
+}
 __device__ __forceinline__ void stpop(float* p, float v) {
 #if LBM_STPOP_CS
     __stcs(p, v);
@@ -565,7 +578,7 @@ struct DomPlanes {
 struct RsOff32 {
     const float* r;
     const Off32& o;
-    __device__ __forceinline__ float at(int dx, int dy, int dz) const { return __ldg(r + o.nb(dx, dy, dz)); }
+    __device__ __forceinline__ float at(int dx, int dy, int dz) const { return ldnow(r + o.nb(dx, dy, dz)); }
 };
 
 template <int Q, int PARITY, bool SOLIDS, class A>
