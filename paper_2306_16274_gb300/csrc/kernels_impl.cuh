@@ -1,6 +1,7 @@
 // Kernels of one lattice; included by kernels_q19.cu / kernels_q27.cu with LBM_Q set.
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -1495,13 +1496,20 @@ cudaError_t LBM_CAT(launch_psi_q, LBM_Q)(const KParams& kp, int parity, int soli
                  : launch_psi_store<false>(g, b, st, kp, parity, solids, B);
 }
 
-// z planes per block: enough blocks for a few waves of resident blocks on 152 SMs
 // z-planes per block of the z-marching kernels.  Blocks of equal size run in waves of
 // (SMs x resident blocks); a last wave that is mostly empty leaves SMs idle, and every chunk
 // costs about h planes' worth of extra time at its start (the psi planes below and at its first
 // plane, the first loads with nothing to overlap them); and blocks differ in duration, which more
 // waves even out.  Over the chunk counts that give at least three waves, the choice minimises
 // (1 + h / zc) x ceil(waves) / waves x (1 + 0.2 / waves) (0.2 fitted to 256^3 sweeps).
+//
+// Domains of fewer than 17 column-planes a resident block have too few planes for three waves of chunks
+// worth their start.  A block's march is then a chain of (zc + 2) planes of a latency L that more blocks on
+// the SM hardly change, and all blocks together need (blocks / SMs) (zc + 1) planes' time t each; with
+// B = (zc + 2) L / t and A the latter, a little more where the last wave is partly empty, the choice minimises
+// max(B, A + 0.35 B).  L / t = 6.1 (D3Q19: 2.1 us over 0.34) and 5 (D3Q27: 2.3 us over 0.46), from sweeps of zc
+// over 16^3 - 112^3.  us a step, the three-wave rule / this one: D3Q19 64^3 13.3 / 12.3, 80^3 25.2 / 22.9,
+// 96^3 31.7 / 30.7; D3Q27 61 x 83 x 70 23.9 / 21.9, 64^3 17.3 / 16.4, 112^3 83.8 / 82.0.
 static int choose_zchunk(const KParams& kp, double h, int nz, int by, int minb) {
     if (kp.zchunk > 0) return kp.zchunk < nz ? kp.zchunk : nz;
     if (nz <= 1) return 1;
@@ -1518,6 +1526,8 @@ static int choose_zchunk(const KParams& kp, double h, int nz, int by, int minb) 
     if (k[0] == key[0] && k[1] == key[1] && k[2] == key[2] && k[3] == key[3]) return cached;
     const double cap = (double)sms * minb;
     const long long cols = (long long)((kp.nx + ZM_BX - 1) / ZM_BX) * ((kp.ny + by - 1) / by);
+    const bool few = (double)cols * nz < 17.0 * cap;
+    const double ratio = LBM_Q == 19 ? 6.1 : 5.0;
     int best = nz;
     double best_cost = 1e300;
     for (int c = 1; c <= nz; ++c) {
@@ -1525,8 +1535,15 @@ static int choose_zchunk(const KParams& kp, double h, int nz, int by, int minb) 
         const int chunks = (nz + zc - 1) / zc;
         if (chunks != c) continue;                 // the same split as a smaller count
         const double waves = (double)(cols * chunks) / cap;
-        if (waves < 3.0 && c < nz) continue;
-        const double cost = (1.0 + h / zc) * std::ceil(waves) / waves * (1.0 + 0.2 / waves);
+        double cost;
+        if (few) {
+            const double B = (zc + 2) * ratio;
+            const double A = (double)(cols * chunks) / sms * (zc + 1) * (1.0 + 0.15 * (std::ceil(waves) / waves - 1.0));
+            cost = std::max(B, A + 0.35 * B);
+        } else {
+            if (waves < 3.0 && c < nz) continue;
+            cost = (1.0 + h / zc) * std::ceil(waves) / waves * (1.0 + 0.2 / waves);
+        }
         if (cost < best_cost - 1e-9) { best_cost = cost; best = zc; }
     }
     for (int i = 0; i < 4; ++i) key[i] = k[i];
