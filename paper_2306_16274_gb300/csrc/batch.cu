@@ -70,7 +70,6 @@ KParams physics_of(const KParams& k) {
     for (float*& q : p.fq) q = nullptr;
     for (float*& q : p.gq) q = nullptr;
     p.zchunk = 0;
-    p.zlo = p.zhi = 0;
     p.paired = p.hx = 0;        // storage layout (FP16 only), not physics
     return p;
 }

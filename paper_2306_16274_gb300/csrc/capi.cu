@@ -1,6 +1,7 @@
 // C ABI of liblbm.so (declared in include/lbm.h): context lifetime, parameter
 // validation and derivation, step sequencing (AA parity), host<->device
 // marshalling, status handling and kernel timing.
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cstdio>
@@ -160,8 +161,6 @@ KParams derive(const lbm_params& p, long long plane) {
     k.gy = (float)p.g[1];
     k.gz = (float)p.g[2];
     k.zchunk = p.zchunk;
-    k.zlo = 0;
-    k.zhi = p.nz;
     return k;
 }
 
@@ -185,6 +184,7 @@ lbm::Bufs bufs(const lbm_ctx* c) {
     b.f = c->f;
     b.psi = c->psi;
     b.nbmask = c->nbmask;
+    b.zmask = c->zmask;
     b.status = c->status;
     b.f16 = c->f16;
     b.paired = c->paired;
@@ -263,35 +263,12 @@ cudaError_t run_onepass(lbm_ctx* c) {
     return e;
 }
 
-// Walls only at the two z ends (the droplet-impact setup): the planes between them need no
-// solid handling, so they take the solid-free kernel and only the two wall planes the solid one.
-bool zwalls_only(const lbm_ctx* c) {
-    return !c->nbmask && !c->kp.wall_x && !c->kp.wall_y && c->kp.wall_z && c->kp.nz >= 3 && !c->onepass;
-}
-
-cudaError_t launch_collide(const lbm_ctx* c, const lbm::KParams& k, int solids) {
-    return c->Q == 19 ? lbm::launch_collide_q19(k, c->parity, solids, bufs(c), c->stream)
-                      : lbm::launch_collide_q27(k, c->parity, solids, bufs(c), c->stream);
-}
-
 cudaError_t run_collide(lbm_ctx* c) {
-    cudaError_t e;
     lbm::KParams k = c->kp;
     k.down = !k.multiphase && !c->f16 ? c->parity : 0;   // without a density pass: against the step before
-    if (zwalls_only(c)) {
-        // each slot is read and written by one cell only, so the three plane ranges are independent
-        k.zlo = 1;
-        k.zhi = k.nz - 1;
-        e = launch_collide(c, k, 0);
-        k.zlo = 0;
-        k.zhi = 1;
-        if (e == cudaSuccess) e = launch_collide(c, k, 1);
-        k.zlo = k.nz - 1;
-        k.zhi = k.nz;
-        if (e == cudaSuccess) e = launch_collide(c, k, 1);
-    } else {
-        e = launch_collide(c, k, has_solids(c));
-    }
+    const int s = has_solids(c);
+    cudaError_t e = c->Q == 19 ? lbm::launch_collide_q19(k, c->parity, s, bufs(c), c->stream)
+                               : lbm::launch_collide_q27(k, c->parity, s, bufs(c), c->stream);
     if (c->f16) c->rs ^= 1;   // the slots are now relative to the densities the collide pass used
     return e;
 }
@@ -468,22 +445,29 @@ lbm_status lbm_init_fields(lbm_ctx* c, const float* rho, const float* u, const u
     }
     if (solid && c->onepass) return fail(c, LBM_ERR_ARG, "onepass contexts take no solid mask");
     if (solid) {
+        const size_t words = (size_t)lbm::solid_plane_words(c->kp) * sizeof(uint32_t);
         if (!c->nbmask) {
             CK(c, cudaMalloc((void**)&c->nbmask, n * sizeof(uint32_t)));
             c->bytes += n * sizeof(uint32_t);
         }
         if (!c->solid_dev) {
-            CK(c, cudaMalloc((void**)&c->solid_dev, n));
+            // (room for the words below; they exceed the mask in domains of a few cells only, far below the
+            // allocator's granularity)
+            CK(c, cudaMalloc((void**)&c->solid_dev, std::max<size_t>(n, words)));
             c->bytes += n;
         }
         CK(c, cudaMemcpyAsync(c->solid_dev, solid, n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                               c->stream));
         CK(c, lbm::launch_nbmask(c->kp, c->Q, c->solid_dev, c->nbmask, c->stream));
+        // the neighbour mask holds all that the steps need of the solid copy: its buffer takes the planes' words
+        c->zmask = reinterpret_cast<uint32_t*>(c->solid_dev);
+        CK(c, c->Q == 19 ? lbm::launch_solid_planes_q19(c->kp, c->nbmask, c->zmask, c->stream)
+                         : lbm::launch_solid_planes_q27(c->kp, c->nbmask, c->zmask, c->stream));
     } else if (c->nbmask) {
         // walls are handled arithmetically; no mask means "no interior solids"
         CK(c, cudaFree(c->nbmask));
         c->bytes -= n * sizeof(uint32_t);
-        c->nbmask = nullptr;
+        c->nbmask = c->zmask = nullptr;
     }
     c->tile_flags.clear();
     set_layout(c, solid != nullptr);
@@ -531,18 +515,6 @@ lbm_status lbm_step(lbm_ctx* c, int32_t n) {
             if (c->timing) CK(c, record(c));
             c->t += 1;
         }
-        return LBM_OK;
-    }
-    if (has_solids(c) && !zwalls_only(c) && !c->timing && !c->f16 && n > 0 &&
-        (unsigned long long)c->Q * (unsigned long long)c->kp.plane <= 0xFFFFFFFFull) {
-        // walls or solids: the tile path, which runs solid-free tiles without solid handling
-        if (!c->self_batch) {
-            lbm_ctx* self[1] = {c};
-            lbm_status bs = lbm_batch_create(self, 1, c->stream, &c->self_batch);
-            if (bs != LBM_OK) return fail(c, bs, std::string("tile path: ") + lbm_last_error(nullptr));
-        }
-        lbm_status bs = lbm_batch_step(c->self_batch, n);
-        if (bs != LBM_OK) return fail(c, bs, std::string("tile path: ") + lbm_batch_last_error(c->self_batch));
         return LBM_OK;
     }
     for (int32_t k = 0; k < n; ++k) {
@@ -655,10 +627,6 @@ lbm_status lbm_set_populations(lbm_ctx* c, const float* f, int on_device) {
 
 lbm_status lbm_set_stream(lbm_ctx* c, void* cuda_stream) {
     if (!c) return LBM_ERR_ARG;
-    if (c->self_batch) {   // bound to the old stream
-        lbm_batch_destroy(c->self_batch);
-        c->self_batch = nullptr;
-    }
     c->stream = (cudaStream_t)cuda_stream;
     return LBM_OK;
 }
@@ -716,7 +684,6 @@ lbm_status lbm_contact(lbm_ctx* c, float rho_threshold, int32_t* out, int on_dev
 
 void lbm_destroy(lbm_ctx* c) {
     if (!c) return;
-    if (c->self_batch) lbm_batch_destroy(c->self_batch);
     if (c->stream || c->f) (void)cudaStreamSynchronize(c->stream);
     for (cudaEvent_t e : c->ev) (void)cudaEventDestroy(e);
     void* ptrs[] = {c->f, c->psi, c->nbmask, c->status, c->partials, c->sums, c->staging, c->solid_dev,

@@ -30,6 +30,7 @@ struct lbm_ctx {
     int rs = 0;
     float* psi = nullptr;        // ncell floats
     uint32_t* nbmask = nullptr;  // ncell words, only when a solid mask was given
+    uint32_t* zmask = nullptr;   // with nbmask: solid_plane_words(kp) words (in solid_dev)
     unsigned* status = nullptr;  // device status word
     double* partials = nullptr;  // moments partial sums (4 per block)
     double* sums = nullptr;      // 4 doubles
@@ -41,9 +42,6 @@ struct lbm_ctx {
     // computed on first use by a multi-domain batch, cleared when the fields are re-initialised
     std::vector<uint8_t> tile_flags;
     int tile_flags_tw = 0, tile_flags_th = 0;   // the column shape tile_flags was computed for
-    // domains with walls or solids step through a one-member batch (created on first use): its
-    // tiles away from solids take the kernels without solid handling
-    lbm_batch* self_batch = nullptr;
     long long partial_blocks = 0;
     // host state
     int parity = 0;              // 0: natural layout, 1: swapped (after an odd number of AA steps)

@@ -16,6 +16,48 @@ namespace {
 
 constexpr int Q = LBM_Q;
 
+// Which planes of a 32 x 4 column hold cells with solid neighbours: all of them in a column at a wall in x
+// or y, the first and the last with walls in z, and those whose bits the mask's words have (one word per
+// column and 32 planes).  Only these take the code with solid tests: in a 127 x 127 x 106 domain with a
+// cylinder on the floor 1 plane in 6.
+struct SolidPlanes {
+    const uint32_t* words = nullptr;   // this column's words, `stride` apart; null: no mask
+    int stride = 0, nz = 0, group = -1;
+    bool side = false, wall_z = false;
+    uint32_t word = 0u;
+    __device__ __forceinline__ SolidPlanes() {}
+    template <class GM>
+    __device__ __forceinline__ SolidPlanes(const GM& g, const uint32_t* zmask, int x0, int y0, int w, int h, int col,
+                                           int ncol)
+        : words(zmask ? zmask + col : nullptr), stride(ncol), nz(g.nz()),
+          side((g.wall_x() && (x0 == 0 || x0 + w >= g.nx())) || (g.wall_y() && (y0 == 0 || y0 + h >= g.ny()))),
+          wall_z(g.wall_z()) {}
+    __device__ __forceinline__ bool at(int z) {
+        if (side || (wall_z && (z == 0 || z == nz - 1))) return true;
+        if (!words) return false;
+        if ((z >> 5) != group) {
+            group = z >> 5;
+            word = __ldg(words + (size_t)group * stride);
+        }
+        return (word >> (z & 31)) & 1u;
+    }
+};
+
+// Marches a chunk [z0, z1) of a column as runs of planes with and without solid neighbours: a run starts
+// its own march (two psi planes and a first plane that nothing overlaps), which only the columns and chunks
+// at solids pay.  The ring is free again for a run once every thread has left the one before it.
+template <class F>
+__device__ __forceinline__ void for_plane_runs(SolidPlanes& sp, int z0, int z1, F&& run) {
+    for (int za = z0; za < z1;) {
+        const bool solids = sp.at(za);
+        int zb = za + 1;
+        while (zb < z1 && sp.at(zb) == solids) ++zb;
+        if (za > z0) __syncthreads();
+        run(solids, za, zb);
+        za = zb;
+    }
+}
+
 // ---- density + psi pass (Sec. II A, Sec. II C): one thread per cell, x fastest
 constexpr int PSI_BX = 32, PSI_BY = 4;
 
@@ -94,17 +136,26 @@ __device__ __forceinline__ int swept_block(int down) {
     return down ? (int)gridDim.z - 1 - (int)blockIdx.z : (int)blockIdx.z;
 }
 
-template <int PARITY, bool SOLIDS, bool F16>
+// MIXED: solid handling in the planes that the column's SolidPlanes name
+template <int PARITY, bool MIXED, bool F16>
 __global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_kernel(KParams kp, float* __restrict__ psi,
                                                             const uint32_t* __restrict__ nbmask, unsigned* status,
                                                             const float* __restrict__ rsrc,
-                                                            float* __restrict__ rdst) {
+                                                            float* __restrict__ rdst,
+                                                            const uint32_t* __restrict__ zmask) {
     const KGeom g{kp};
     const PlanePtrsT<typename std::conditional<F16, __half, float>::type> addr{kp};
     const int z = swept_block(kp.down);
     dep_wait();
-    psi_column<PARITY, SOLIDS, F16>(kp, g, addr, psi, nbmask, status, blockIdx.x * PSI_BX + threadIdx.x,
-                                    blockIdx.y * PSI_BY + threadIdx.y, z, z + 1, rsrc, rdst);
+    const int x0 = blockIdx.x * PSI_BX, y0 = blockIdx.y * PSI_BY;
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+    // (the FP16 store's densities are summed by one code throughout a domain with solids: the compiler fuses
+    // the products of the two forms differently)
+    if (MIXED && (F16 || SolidPlanes(g, zmask, x0, y0, PSI_BX, PSI_BY, blockIdx.y * gridDim.x + blockIdx.x,
+                                     gridDim.x * gridDim.y).at(z)))
+        psi_column<PARITY, true, F16>(kp, g, addr, psi, nbmask, status, x, y, z, z + 1, rsrc, rdst);
+    else
+        psi_column<PARITY, false, F16>(kp, g, addr, psi, nbmask, status, x, y, z, z + 1, rsrc, rdst);
 }
 
 
@@ -236,19 +287,57 @@ __device__ __forceinline__ void put_psi_plane(float* slot, const float (&v)[TS::
 #define LBM_ZM_PREFETCH 1
 #endif
 
+// the parts of a mixed tile's cell (SOLIDS == 2 below): its populations and solid bits, returning whether
+// the tile has solid neighbours in plane z ...
+template <int PARITY, class GM, class A>
+__device__ __forceinline__ bool gather_mixed(const GM& g, const A& addr, const Off32& o,
+                                             const uint32_t* __restrict__ nbmask, SolidPlanes& sp, int x, int y, int z,
+                                             uint32_t& bits, float (&p)[Q]) {
+    if (sp.at(z)) {
+        bits = solid_bits32<Q>(g, nbmask, o.c, x, y, z);
+        if (!(bits & 1u)) gather32<Q, PARITY, true>(addr, o, bits, p);
+        return true;
+    }
+    bits = 0u;
+    gather32<Q, PARITY, false>(addr, o, 0u, p);
+    return false;
+}
+// ... and its forces (FP16: after de-normalising the populations) from ring planes j, j + 1, j + 2
+template <class TS>
+struct RingAt {
+    float (*psi)[TS::RP], (*rho)[TS::RP];
+    int j, lc;
+};
+template <bool SOLIDS, bool MULTIPHASE, bool F16, class TS>
+__device__ __forceinline__ void cell_forces(const KParams& kp, float (&p)[Q], const RingAt<TS>& r, uint32_t bits,
+                                            Forces& Fo) {
+    const int a = r.j & 3, b = (r.j + 1) & 3, c = (r.j + 2) & 3;
+    if (F16) denorm<Q, SOLIDS>(p, bits, RsRing{&r.rho[a][r.lc], &r.rho[b][r.lc], &r.rho[c][r.lc], TS::RX});
+    if (MULTIPHASE) {
+        Fo = stencil_forces3<Q, SOLIDS>(kp, &r.psi[a][r.lc], &r.psi[b][r.lc], &r.psi[c][r.lc], TS::RX, bits);
+    } else {
+        Fo.fx = Fo.fy = Fo.fz = 0.f;
+        Fo.qxx = Fo.qyy = Fo.qzz = Fo.qxy = Fo.qxz = Fo.qyz = 0.f;
+        Fo.s2 = 0.f;
+    }
+}
+
 // One tile: cells [x0, x0+TS::BX) x [y0, y0+TS::BY) marching through planes [z0, z0+zchunk); `addr`
 // locates population planes.  F16 (shifted FP16 store): the densities the slots were written
 // with (rsrc) follow the march in a second shared ring `rring`; outputs are written relative
 // to the cell's current density rown.
+// SOLIDS: 0 no cell of the tile has a solid neighbour, 1 every cell is tested, 2 the cells of the planes that
+// sp names (the march switches from plane to plane; only for whole-grid tiles).
 // PSI_PF: the psi (and FP16 density) ring planes are loaded into registers one plane ahead and
 // stored into the ring at the next plane (all but the multi-domain kernels' solid tiles, which
 // have no registers to spare and load each plane just before its barrier).
-template <class TS, int PARITY, bool SOLIDS, bool MULTIPHASE, bool F16, bool PSI_PF, class GM, class A,
+template <class TS, int PARITY, int SOLIDS, bool MULTIPHASE, bool F16, bool PSI_PF, class GM, class A,
           bool FLAT = false>
 __device__ __forceinline__ void collide_tile(const KParams& kp, const GM& g, const A& addr, const float* __restrict__ psi,
                                              const uint32_t* __restrict__ nbmask, unsigned* status, int x0, int y0,
                                              int z0, int zchunk, int zmax, float (*ring)[TS::RP], float (*rring)[TS::RP],
-                                             const float* __restrict__ rsrc, const float* __restrict__ rown) {
+                                             const float* __restrict__ rsrc, const float* __restrict__ rown,
+                                             SolidPlanes sp = SolidPlanes()) {
     // FLAT: the block has another shape with as many threads (a narrow multi-domain tile); its threads
     // take the tile's cells in row-major order
     const int tid = FLAT ? (int)(threadIdx.x + blockDim.x * threadIdx.y) : (int)(threadIdx.x + TS::BX * threadIdx.y);
@@ -287,10 +376,15 @@ __device__ __forceinline__ void collide_tile(const KParams& kp, const GM& g, con
     // chunk's start-up waits for one round trip instead of two
     float pn[Q];
     uint32_t bits_n = 0u;
+    bool near_n = false;   // SOLIDS == 2: the tile has solid neighbours in the plane that pn belongs to
     if (act_xy) {
         set_plane(o, z0, nz, nxy);
-        bits_n = SOLIDS ? solid_bits32<Q>(g, nbmask, o.c, x, y, z0) : 0u;
-        if (!(bits_n & 1u)) gather32<Q, PARITY, SOLIDS>(addr, o, bits_n, pn);
+        if constexpr (SOLIDS == 2) {
+            near_n = gather_mixed<PARITY>(g, addr, o, nbmask, sp, x, y, z0, bits_n, pn);
+        } else {
+            bits_n = SOLIDS ? solid_bits32<Q>(g, nbmask, o.c, x, y, z0) : 0u;
+            if (!(bits_n & 1u)) gather32<Q, PARITY, SOLIDS>(addr, o, bits_n, pn);
+        }
     }
 #endif
     float pv[TS::SLOTS], rv[TS::SLOTS];
@@ -326,52 +420,121 @@ __device__ __forceinline__ void collide_tile(const KParams& kp, const GM& g, con
 #pragma unroll
         for (int i = 0; i < Q; ++i) p[i] = pn[i];
         const uint32_t bits = bits_n;
+        [[maybe_unused]] const bool near = near_n;
         if (z + 1 < zend) {
             set_plane(o, z + 1, nz, nxy);
-            bits_n = SOLIDS ? solid_bits32<Q>(g, nbmask, o.c, x, y, z + 1) : 0u;
-            if (!(bits_n & 1u)) gather32<Q, PARITY, SOLIDS>(addr, o, bits_n, pn);
+            if constexpr (SOLIDS == 2) {
+                near_n = gather_mixed<PARITY>(g, addr, o, nbmask, sp, x, y, z + 1, bits_n, pn);
+            } else {
+                bits_n = SOLIDS ? solid_bits32<Q>(g, nbmask, o.c, x, y, z + 1) : 0u;
+                if (!(bits_n & 1u)) gather32<Q, PARITY, SOLIDS>(addr, o, bits_n, pn);
+            }
         }
         set_plane(o, z, nz, nxy);
         if (bits & 1u) continue;
 #else
+        static_assert(SOLIDS != 2, "mixed tiles gather a plane ahead");
         set_plane(o, z, nz, nxy);
         const uint32_t bits = SOLIDS ? solid_bits32<Q>(g, nbmask, o.c, x, y, z) : 0u;
         if (bits & 1u) continue;
         float p[Q];
         gather32<Q, PARITY, SOLIDS>(addr, o, bits, p);
 #endif
-        if (F16) denorm<Q, SOLIDS>(p, bits, RsRing{&rring[j & 3][lc], &rring[(j + 1) & 3][lc],
-                                                    &rring[(j + 2) & 3][lc], TS::RX});
-        Forces Fo;
-        if (MULTIPHASE) {
-            Fo = stencil_forces3<Q, SOLIDS>(kp, &ring[j & 3][lc], &ring[(j + 1) & 3][lc], &ring[(j + 2) & 3][lc],
-                                            TS::RX, bits);
-        } else {
-            Fo.fx = Fo.fy = Fo.fz = 0.f;
-            Fo.qxx = Fo.qyy = Fo.qzz = Fo.qxy = Fo.qxz = Fo.qyz = 0.f;
-            Fo.s2 = 0.f;
-        }
         float rho, ux, uy, uz;
-        collide<Q>(kp, p, Fo, rho, ux, uy, uz);
+        if constexpr (SOLIDS == 2) {
+            // both ways of a cell up to its forces; with the FP16 store the collision too, since the compiler
+            // fuses the de-normalising products into it
+            const RingAt<TS> at{ring, rring, j, lc};
+            Forces Fo;
+            if (near) {
+                cell_forces<true, MULTIPHASE, F16>(kp, p, at, bits, Fo);
+                if (F16) collide<Q>(kp, p, Fo, rho, ux, uy, uz);
+            } else {
+                cell_forces<false, MULTIPHASE, F16>(kp, p, at, 0u, Fo);
+                if (F16) collide<Q>(kp, p, Fo, rho, ux, uy, uz);
+            }
+            if (!F16) collide<Q>(kp, p, Fo, rho, ux, uy, uz);
+        } else {
+            if (F16) denorm<Q, SOLIDS>(p, bits, RsRing{&rring[j & 3][lc], &rring[(j + 1) & 3][lc],
+                                                        &rring[(j + 2) & 3][lc], TS::RX});
+            Forces Fo;
+            if (MULTIPHASE) {
+                Fo = stencil_forces3<Q, SOLIDS>(kp, &ring[j & 3][lc], &ring[(j + 1) & 3][lc], &ring[(j + 2) & 3][lc],
+                                                TS::RX, bits);
+            } else {
+                Fo.fx = Fo.fy = Fo.fz = 0.f;
+                Fo.qxx = Fo.qyy = Fo.qzz = Fo.qxy = Fo.qxz = Fo.qyz = 0.f;
+                Fo.s2 = 0.f;
+            }
+            collide<Q>(kp, p, Fo, rho, ux, uy, uz);
+        }
         if (!(rho > 0.0f) || !(fabsf(ux) + fabsf(uy) + fabsf(uz) < 1e30f)) atomicOr(status, ST_UNSTABLE);
         if (F16) normalize<Q>(p, ldnow(rown + o.c));
-        store32<Q, PARITY, SOLIDS>(addr, o, bits, p);
+        if constexpr (SOLIDS == 2) {
+            if (near) store32<Q, PARITY, true>(addr, o, bits, p);
+            else store32<Q, PARITY, false>(addr, o, 0u, p);
+        } else {
+            store32<Q, PARITY, SOLIDS>(addr, o, bits, p);
+        }
     }
 }
 
-template <int PARITY, bool SOLIDS, bool MULTIPHASE, bool F16>
-__global__ void __launch_bounds__(ZmTile::NT, ZM_MINB) collide_kernel(const KParams kp, const float* __restrict__ psi,
+// Planes with solid neighbours of one tile, as a function of its own: its registers (it spills at this
+// kernel's limit) and its code stay apart from those of the tiles without.
+template <int PARITY, bool MULTIPHASE, bool F16>
+__device__ __noinline__ void collide_tile_near(const KParams& kp, const float* psi, const uint32_t* nbmask,
+                                               unsigned* status, int x0, int y0, int z0, int zend,
+                                               float (*ring)[ZmTile::RP], const float* rsrc, const float* rown) {
+    const KGeom g{kp};
+    const PlanePtrsT<typename std::conditional<F16, __half, float>::type> addr{kp};
+    collide_tile<ZmTile, PARITY, true, MULTIPHASE, F16, true>(kp, g, addr, psi, nbmask, status, x0, y0, z0, zend - z0,
+                                                              zend, ring, ring + 4, rsrc, rown);
+}
+
+// NEAR: which cells have solid neighbours -- NEAR_NONE: none; NEAR_ENDS: those of the first and the last plane
+// (walls in z), which have blocks of their own (short ones, the grid's last); NEAR_SOME: those of the
+// planes that the column's SolidPlanes name.
+// us a step: walls in z as three launches / as one, D3Q19 64^3 21.0 / 13.7, 200 x 200 x 100 173.6 / 166.8 (FP16
+// store 226.5 / 214.6, 400 x 400 x 200 1446 / 1447), D3Q27 200 x 200 x 100 241.8 / 234.2.  A cylinder on the floor
+// as two launches a pass over tile lists, replayed from a graph / as one kernel: D3Q19 127 x 127 x 106 92.5 /
+// 77.8, 256^3 746 / 672, D3Q27 127 x 127 x 106 130.9 / 107.1.  (As a march cut into runs with and without solids,
+// each through its own copy of the tile: 87.9, 709 and 127.6 us; registers spill in the plain copy.)
+enum { NEAR_NONE = 0, NEAR_ENDS = 1, NEAR_SOME = 2 };
+template <int PARITY, int NEAR, bool MULTIPHASE, bool F16>
+__global__ void __launch_bounds__(ZmTile::NT, ZM_MINB) collide_kernel(const __grid_constant__ KParams kp,
+                                                                const float* __restrict__ psi,
                                                                 const uint32_t* __restrict__ nbmask,
                                                                 unsigned* status, int zchunk,
                                                                 const float* __restrict__ rsrc,
-                                                                const float* __restrict__ rown) {
+                                                                const float* __restrict__ rown,
+                                                                const uint32_t* __restrict__ zmask) {
+    static_assert(ZM_BX == PSI_BX && ZM_BY == PSI_BY, "both passes go by the same columns' words");
     __shared__ float ring[F16 ? 8 : 4][ZmTile::RP];
     const KGeom g{kp};
     const PlanePtrsT<typename std::conditional<F16, __half, float>::type> addr{kp};
+    const int x0 = blockIdx.x * ZM_BX, y0 = blockIdx.y * ZM_BY;
     dep_wait();
-    collide_tile<ZmTile, PARITY, SOLIDS, MULTIPHASE, F16, true>(kp, g, addr, psi, nbmask, status, blockIdx.x * ZM_BX,
-                                                        blockIdx.y * ZM_BY, kp.zlo + swept_block(kp.down) * zchunk,
-                                                        zchunk, kp.zhi, ring, ring + 4, rsrc, rown);
+    if (NEAR == NEAR_NONE) {
+        collide_tile<ZmTile, PARITY, false, MULTIPHASE, F16, true>(kp, g, addr, psi, nbmask, status, x0, y0,
+                                                                   swept_block(kp.down) * zchunk, zchunk, kp.nz, ring,
+                                                                   ring + 4, rsrc, rown);
+    } else if (NEAR == NEAR_ENDS) {
+        const int chunks = (int)gridDim.z - 2, k = (int)blockIdx.z;
+        if (k >= chunks) {
+            const int z = k == chunks ? 0 : kp.nz - 1;
+            collide_tile_near<PARITY, MULTIPHASE, F16>(kp, psi, nbmask, status, x0, y0, z, z + 1, ring, rsrc, rown);
+        } else {
+            const int z0 = 1 + (kp.down ? chunks - 1 - k : k) * zchunk;
+            collide_tile<ZmTile, PARITY, false, MULTIPHASE, F16, true>(kp, g, addr, psi, nbmask, status, x0, y0,
+                                                                       z0, zchunk, kp.nz - 1, ring, ring + 4, rsrc,
+                                                                       rown);
+        }
+    } else {
+        const SolidPlanes sp(g, zmask, x0, y0, ZM_BX, ZM_BY, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+        collide_tile<ZmTile, PARITY, 2, MULTIPHASE, F16, true>(kp, g, addr, psi, nbmask, status, x0, y0,
+                                                               swept_block(kp.down) * zchunk, zchunk, kp.nz, ring,
+                                                               ring + 4, rsrc, rown, sp);
+    }
 }
 
 // ---- shifted FP16 store in the x-paired layout (KParams::paired: even nx, x periodic, no solid
@@ -610,21 +773,19 @@ __global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_pair_kernel(KParams kp, f
     }
 }
 
+// Planes [z0, zend) of one tile of pairs; ring: psi (low cells, high cells), rring: the densities the
+// slots were written with.
 template <int PARITY, bool SOLIDS, bool MULTIPHASE>
-__global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const KParams kp, const float* __restrict__ psi,
-                                                                     unsigned* status, int zchunk,
-                                                                     const float* __restrict__ rsrc,
-                                                                     const float* __restrict__ rown) {
-    __shared__ float ring[4][2][PR_RP];    // psi (low cells, high cells)
-    __shared__ float rring[4][2][PR_RP];   // densities the slots were written with
+__device__ __forceinline__ void collide_pair_tile(const KParams& kp, const float* __restrict__ psi, unsigned* status, int z0,
+                                                  int zend, const float* __restrict__ rsrc,
+                                                  const float* __restrict__ rown, float (*ring)[2][PR_RP],
+                                                  float (*rring)[2][PR_RP]) {
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + PR_BX * ty;
     const int hx = kp.hx, nx = kp.nx, ny = kp.ny, nz = kp.nz;
     const int w0 = blockIdx.x * PR_BX, y0 = blockIdx.y * PR_BY;
     const int w = w0 + tx, y = y0 + ty;
     const bool act = w < hx && y < ny;
     const uint32_t nxy = (uint32_t)nx * (uint32_t)ny, wpl = (uint32_t)hx * (uint32_t)ny;
-    const int z0 = kp.zlo + swept_block(kp.down) * zchunk;
-    const int zend = min(z0 + zchunk, kp.zhi);
     const KGeom g{kp};
     const WordPlanes addr{kp};
 
@@ -634,7 +795,6 @@ __global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const KPar
     const uint32_t selL = w == 0 ? PERM_SWAP : PERM_KEEP, selR = w == hx - 1 ? PERM_SWAP : PERM_KEEP;
     const uint32_t rowA = (uint32_t)(y < ny ? y : 0) * (uint32_t)nx + (uint32_t)(w < hx ? w : 0);   // low cell in its plane
 
-    dep_wait();
     // words and own densities of the first plane, then of plane z+1 while plane z is computed
     uint32_t wn[Q];
     float rn[2] = {0.0f, 0.0f};
@@ -721,6 +881,49 @@ __global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const KPar
             }
         }
         store_pair<PARITY, SOLIDS>(addr, o, bits, selL, selR, wv);
+    }
+}
+
+template <int PARITY, bool MULTIPHASE>
+__device__ __noinline__ void collide_pair_tile_near(const KParams& kp, const float* psi, unsigned* status, int z0, int zend,
+                                                    const float* rsrc, const float* rown, float (*ring)[2][PR_RP],
+                                                    float (*rring)[2][PR_RP]) {
+    collide_pair_tile<PARITY, true, MULTIPHASE>(kp, psi, status, z0, zend, rsrc, rown, ring, rring);
+}
+
+// NEAR as in collide_kernel (no mask in this layout: only cells at walls in y and z have solid neighbours)
+template <int PARITY, int NEAR, bool MULTIPHASE>
+__global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const __grid_constant__ KParams kp,
+                                                                     const float* __restrict__ psi,
+                                                                     unsigned* status, int zchunk,
+                                                                     const float* __restrict__ rsrc,
+                                                                     const float* __restrict__ rown) {
+    __shared__ float ring[4][2][PR_RP];
+    __shared__ float rring[4][2][PR_RP];
+    dep_wait();
+    if (NEAR == NEAR_NONE) {
+        const int z0 = swept_block(kp.down) * zchunk;
+        collide_pair_tile<PARITY, false, MULTIPHASE>(kp, psi, status, z0, min(z0 + zchunk, kp.nz), rsrc, rown, ring,
+                                                     rring);
+    } else if (NEAR == NEAR_ENDS) {
+        const int chunks = (int)gridDim.z - 2, k = (int)blockIdx.z;
+        if (k >= chunks) {
+            const int z = k == chunks ? 0 : kp.nz - 1;
+            collide_pair_tile_near<PARITY, MULTIPHASE>(kp, psi, status, z, z + 1, rsrc, rown, ring, rring);
+        } else {
+            const int z0 = 1 + (kp.down ? chunks - 1 - k : k) * zchunk;
+            collide_pair_tile<PARITY, false, MULTIPHASE>(kp, psi, status, z0, min(z0 + zchunk, kp.nz - 1), rsrc, rown,
+                                                         ring, rring);
+        }
+    } else {
+        const int z0 = swept_block(kp.down) * zchunk;
+        SolidPlanes sp(KGeom{kp}, nullptr, 0, blockIdx.y * PR_BY, 0, PR_BY, 0, 0);
+        for_plane_runs(sp, z0, min(z0 + zchunk, kp.nz), [&](bool solids, int za, int zb) {
+            if (solids)
+                collide_pair_tile_near<PARITY, MULTIPHASE>(kp, psi, status, za, zb, rsrc, rown, ring, rring);
+            else
+                collide_pair_tile<PARITY, false, MULTIPHASE>(kp, psi, status, za, zb, rsrc, rown, ring, rring);
+        });
     }
 }
 
@@ -1087,6 +1290,24 @@ __global__ void __launch_bounds__(BatchTileShape<S>::NT, batch_minb<S>()) collid
                                                                     nullptr);
 }
 
+// One word per 32 x 4 column and 32 planes: bit k set if a cell of the column in plane 32 g + k is solid or has
+// a solid neighbour (SolidPlanes).  A block per word.
+__global__ void __launch_bounds__(PSI_BX * PSI_BY) solid_planes_kernel(const KParams kp,
+                                                                     const uint32_t* __restrict__ nbmask,
+                                                                     uint32_t* __restrict__ zmask) {
+    const int x = blockIdx.x * PSI_BX + threadIdx.x, y = blockIdx.y * PSI_BY + threadIdx.y;
+    uint32_t word = 0u;
+    for (int k = 0; k < 32; ++k) {
+        const int z = 32 * blockIdx.z + k;
+        bool any = false;
+        if (x < kp.nx && y < kp.ny && z < kp.nz)
+            any = nbmask[((long long)z * kp.ny + y) * kp.nx + x] != 0u;
+        if (__syncthreads_or(any)) word |= 1u << k;
+    }
+    if (threadIdx.x == 0 && threadIdx.y == 0)
+        zmask[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = word;
+}
+
 // ---- initialisation: f_bar = M^-1 m^eq(rho, u) (Eq. e13), natural layout
 // F16: slot i of x is written relative to the density of x - e_i (x itself where that neighbour
 // is solid), the cell that writes it in the AA streaming; rdst receives the initial densities.
@@ -1387,41 +1608,46 @@ cudaError_t launch_dep(void (*kernel)(KA...), dim3 g, dim3 b, cudaStream_t st, A
 #ifndef LBM_ZM_CARVEOUT
 #define LBM_ZM_CARVEOUT -1
 #endif
-template <int PARITY, bool SOLIDS, bool MULTIPHASE, bool F16>
+template <int PARITY, int NEAR, bool MULTIPHASE, bool F16>
 cudaError_t launch_collide_variant(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, const Bufs& B, int zc) {
     if (LBM_ZM_CARVEOUT >= 0) {
         static bool configured = false;
         if (!configured) {
-            cudaError_t e = cudaFuncSetAttribute(collide_kernel<PARITY, SOLIDS, MULTIPHASE, F16>,
+            cudaError_t e = cudaFuncSetAttribute(collide_kernel<PARITY, NEAR, MULTIPHASE, F16>,
                                                  cudaFuncAttributePreferredSharedMemoryCarveout, LBM_ZM_CARVEOUT);
             if (e != cudaSuccess) return e;
             configured = true;
         }
     }
-    return launch_dep(collide_kernel<PARITY, SOLIDS, MULTIPHASE, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, zc, B.rsrc, B.rnew);
+    return launch_dep(collide_kernel<PARITY, NEAR, MULTIPHASE, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, zc, B.rsrc, B.rnew, B.zmask);
 }
 
-template <bool F16>
-cudaError_t launch_collide_store(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, const Bufs& B, int zc, int key) {
-    switch (key) {
-        case 0: return launch_collide_variant<0, false, false, F16>(g, b, st, kp, B, zc);
-        case 1: return launch_collide_variant<0, false, true, F16>(g, b, st, kp, B, zc);
-        case 2: return launch_collide_variant<0, true, false, F16>(g, b, st, kp, B, zc);
-        case 3: return launch_collide_variant<0, true, true, F16>(g, b, st, kp, B, zc);
-        case 4: return launch_collide_variant<1, false, false, F16>(g, b, st, kp, B, zc);
-        case 5: return launch_collide_variant<1, false, true, F16>(g, b, st, kp, B, zc);
-        case 6: return launch_collide_variant<1, true, false, F16>(g, b, st, kp, B, zc);
-        default: return launch_collide_variant<1, true, true, F16>(g, b, st, kp, B, zc);
-    }
+template <int NEAR, bool F16>
+cudaError_t launch_collide_store(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, const Bufs& B, int zc, int parity) {
+    if (parity == 0)
+        return kp.multiphase ? launch_collide_variant<0, NEAR, true, F16>(g, b, st, kp, B, zc)
+                             : launch_collide_variant<0, NEAR, false, F16>(g, b, st, kp, B, zc);
+    return kp.multiphase ? launch_collide_variant<1, NEAR, true, F16>(g, b, st, kp, B, zc)
+                         : launch_collide_variant<1, NEAR, false, F16>(g, b, st, kp, B, zc);
+}
+
+template <int NEAR>
+cudaError_t launch_collide_pairs(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, const Bufs& B, int zc, int parity) {
+    const float *r0 = B.rsrc, *r1 = B.rnew;
+    if (parity == 0)
+        return kp.multiphase ? launch_dep(collide_pair_kernel<0, NEAR, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1)
+                             : launch_dep(collide_pair_kernel<0, NEAR, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+    return kp.multiphase ? launch_dep(collide_pair_kernel<1, NEAR, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1)
+                         : launch_dep(collide_pair_kernel<1, NEAR, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
 }
 
 template <bool F16>
 cudaError_t launch_psi_store(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, int parity, int solids, const Bufs& B) {
-    if (parity == 2) return launch_dep(psi_kernel<2, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    if (parity == 0 && !solids) return launch_dep(psi_kernel<0, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    if (parity == 0) return launch_dep(psi_kernel<0, true, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    if (!solids) return launch_dep(psi_kernel<1, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
-    return launch_dep(psi_kernel<1, true, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew);
+    if (parity == 2) return launch_dep(psi_kernel<2, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew, B.zmask);
+    if (parity == 0 && !solids) return launch_dep(psi_kernel<0, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew, B.zmask);
+    if (parity == 0) return launch_dep(psi_kernel<0, true, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew, B.zmask);
+    if (!solids) return launch_dep(psi_kernel<1, false, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew, B.zmask);
+    return launch_dep(psi_kernel<1, true, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, B.rsrc, B.rnew, B.zmask);
 }
 
 template <bool F16>
@@ -1551,38 +1777,29 @@ static int choose_zchunk(const KParams& kp, double h, int nz, int by, int minb) 
     return best;
 }
 
-// over the planes [zlo, zhi) the whole-grid collide kernels march through
-static int collide_zchunk(const KParams& kp) { return choose_zchunk(kp, 1.0, kp.zhi - kp.zlo, ZM_BY, ZM_MINB); }
-
 cudaError_t LBM_CAT(launch_collide_q, LBM_Q)(const KParams& kp, int parity, int solids, const Bufs& B,
                                              cudaStream_t st) {
-    if (B.paired) {
-        // tiles of 32 pairs: the z-chunk choice counts columns of hx words
-        KParams kw = kp;
-        kw.nx = kp.hx;
-        const int planes = kp.zhi - kp.zlo;
-        const int zc = choose_zchunk(kw, 1.0, planes, PR_BY, PR_MINB);
-        const dim3 g((kp.hx + PR_BX - 1) / PR_BX, (kp.ny + PR_BY - 1) / PR_BY, (planes + zc - 1) / zc), b(PR_BX, PR_BY);
-        const int key = parity * 4 + (solids ? 2 : 0) + (kp.multiphase ? 1 : 0);
-        const float* r0 = B.rsrc;
-        const float* r1 = B.rnew;
-        switch (key) {
-            case 0: return launch_dep(collide_pair_kernel<0, false, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-            case 1: return launch_dep(collide_pair_kernel<0, false, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-            case 2: return launch_dep(collide_pair_kernel<0, true, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-            case 3: return launch_dep(collide_pair_kernel<0, true, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-            case 4: return launch_dep(collide_pair_kernel<1, false, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-            case 5: return launch_dep(collide_pair_kernel<1, false, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-            case 6: return launch_dep(collide_pair_kernel<1, true, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-            default: return launch_dep(collide_pair_kernel<1, true, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-        }
-    }
-    const int zc = collide_zchunk(kp);
-    const int planes = kp.zhi - kp.zlo;
-    const dim3 g((kp.nx + ZM_BX - 1) / ZM_BX, (kp.ny + ZM_BY - 1) / ZM_BY, (planes + zc - 1) / zc), b(ZM_BX, ZM_BY);
-    const int key = parity * 4 + (solids ? 2 : 0) + (kp.multiphase ? 1 : 0);
-    return B.f16 ? launch_collide_store<true>(g, b, st, kp, B, zc, key)
-                 : launch_collide_store<false>(g, b, st, kp, B, zc, key);
+    // walls only at the two z ends: their planes apart, the planes between in the plain kernel's way
+    const bool ends = solids && !B.nbmask && !kp.wall_x && !kp.wall_y && kp.nz >= 3;
+    const int near = !solids ? NEAR_NONE : (ends ? NEAR_ENDS : NEAR_SOME);
+    const int planes = kp.nz - (ends ? 2 : 0);
+    KParams kw = kp;   // pairs: tiles of 32 words, so the z-chunk choice counts columns of hx words
+    if (B.paired) kw.nx = kp.hx;
+    const int zc = B.paired ? choose_zchunk(kw, 1.0, planes, PR_BY, PR_MINB) : choose_zchunk(kp, 1.0, planes, ZM_BY, ZM_MINB);
+    static_assert(PR_BX == ZM_BX && PR_BY == ZM_BY, "one grid for both");
+    const dim3 g((kw.nx + ZM_BX - 1) / ZM_BX, (kp.ny + ZM_BY - 1) / ZM_BY, (planes + zc - 1) / zc + (ends ? 2 : 0)),
+        b(ZM_BX, ZM_BY);
+    if (B.paired)
+        return near == NEAR_NONE   ? launch_collide_pairs<NEAR_NONE>(g, b, st, kp, B, zc, parity)
+               : near == NEAR_ENDS ? launch_collide_pairs<NEAR_ENDS>(g, b, st, kp, B, zc, parity)
+                                   : launch_collide_pairs<NEAR_SOME>(g, b, st, kp, B, zc, parity);
+    if (B.f16)
+        return near == NEAR_NONE   ? launch_collide_store<NEAR_NONE, true>(g, b, st, kp, B, zc, parity)
+               : near == NEAR_ENDS ? launch_collide_store<NEAR_ENDS, true>(g, b, st, kp, B, zc, parity)
+                                   : launch_collide_store<NEAR_SOME, true>(g, b, st, kp, B, zc, parity);
+    return near == NEAR_NONE   ? launch_collide_store<NEAR_NONE, false>(g, b, st, kp, B, zc, parity)
+           : near == NEAR_ENDS ? launch_collide_store<NEAR_ENDS, false>(g, b, st, kp, B, zc, parity)
+                               : launch_collide_store<NEAR_SOME, false>(g, b, st, kp, B, zc, parity);
 }
 
 cudaError_t LBM_CAT(launch_collide_batch_q, LBM_Q)(const KParams& phys, const BatchDomTable& doms,
@@ -1691,6 +1908,13 @@ cudaError_t LBM_CAT(launch_pull_store_q, LBM_Q)(const KParams& kp, const float* 
     return cudaGetLastError();
 }
 
+
+cudaError_t LBM_CAT(launch_solid_planes_q, LBM_Q)(const KParams& kp, const uint32_t* nbmask, uint32_t* zmask,
+                                                  cudaStream_t st) {
+    const dim3 g((kp.nx + PSI_BX - 1) / PSI_BX, (kp.ny + PSI_BY - 1) / PSI_BY, (kp.nz + 31) / 32);
+    solid_planes_kernel<<<g, dim3(PSI_BX, PSI_BY), 0, st>>>(kp, nbmask, zmask);
+    return cudaGetLastError();
+}
 
 cudaError_t LBM_CAT(launch_init_q, LBM_Q)(const KParams& kp, const Bufs& B, const float* rho, const float* u,
                                           cudaStream_t st) {

@@ -42,7 +42,6 @@ struct KParams {
     float gx, gy, gz;             // body force per unit mass
     float* fq[27];                // base of population plane i (f + i * plane); cells < 2^31
     int zchunk;                   // z planes per collide block (0 = automatic)
-    int zlo, zhi;                 // planes [zlo, zhi) the whole-grid collide kernels march through
     int down;                     // 1: the launch takes the planes from the top down
     float* gq[27];                // one-pass layout: planes of the copy the step writes
     // shifted FP16 store in the x-paired layout (even nx, x periodic, no solid mask): word w of a
@@ -117,6 +116,7 @@ struct Bufs {
     void* f;
     float* psi;
     const uint32_t* nbmask;
+    const uint32_t* zmask;        // with nbmask: planes with solid neighbours per column (SolidPlanes)
     unsigned* status;
     int f16;
     int paired;                   // f16 in the x-paired layout (KParams::paired)
@@ -131,6 +131,8 @@ struct Bufs {
                                 cudaStream_t st);                                                   \
     cudaError_t launch_collide_q##Q(const KParams& kp, int parity, int solids, const Bufs& B,       \
                                     cudaStream_t st);                                               \
+    cudaError_t launch_solid_planes_q##Q(const KParams& kp, const uint32_t* nbmask, uint32_t* zmask, \
+                                         cudaStream_t st);                                           \
     cudaError_t launch_init_q##Q(const KParams& kp, const Bufs& B, const float* rho, const float* u, \
                                  cudaStream_t st);                                                  \
     cudaError_t launch_f16_restore_q##Q(const KParams& kp, const Bufs& B, const float* fin,         \
@@ -159,6 +161,11 @@ struct Bufs {
 
 LBM_DECLARE_LAUNCHERS(19)
 LBM_DECLARE_LAUNCHERS(27)
+
+// Words of a domain's zmask: one per 32 x 4 column and 32 planes.
+inline long long solid_plane_words(const KParams& kp) {
+    return (long long)((kp.nx + 31) / 32) * ((kp.ny + 3) / 4) * ((kp.nz + 31) / 32);
+}
 
 // Lattice-independent kernels (capi.cu)
 cudaError_t launch_nbmask(const KParams& kp, int Q, const uint8_t* solid, uint32_t* nbmask, cudaStream_t st);
