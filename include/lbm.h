@@ -248,14 +248,13 @@ void lbm_destroy(lbm_ctx* ctx);
  * tiles (32 x 4 columns by default, see LBM_BATCH_SHAPES) and runs of z planes; a
  * tile whose cells have no solid
  * neighbour (mask or wall) goes to a group without solid handling.  Groups are
- * keyed by (lattice, solid handling, physical parameters); each time step costs,
- * per group and per 64 members, one collide-stream launch and one density/psi
- * launch whose blocks are tiles of all those members, and the groups of one pass
- * run concurrently.  Per cell the arithmetic is the single-domain kernels', so
+ * keyed by (lattice, solid handling, physical parameters); the groups of one lattice
+ * and physics are stepped together: each time step costs, per 64 of their members, one
+ * collide-stream launch and one density/psi launch whose blocks are tiles of all those
+ * members.  Members of different lattices or physics are stepped side by side.
+ * Per cell the arithmetic is the single-domain kernels', so
  * every member evolves bitwise as if stepped alone.  Runs of steps are replayed
- * from one CUDA graph (a device-side loop), so n steps cost one graph launch.
- * lbm_step itself takes this path (a batch of one) for a domain with walls or
- * solids, unless kernel timing is on.
+ * from CUDA graphs.
  *
  * lbm_batch_create: ctxs are n >= 1 distinct, initialised contexts on the current
  *   device that have taken the same number of steps modulo 2, each holding fewer
@@ -271,17 +270,17 @@ void lbm_destroy(lbm_ctx* ctx);
  *   advances their step counters.  LBM_ERR_STATE if members were stepped apart.
  * lbm_batch_sync: waits and returns the first sticky member error (lbm_sync).
  * lbm_batch_tune: autotunes each group's launch shape on the live state, in two
- *   stages, by timing the collide launches of every group for trial_steps steps:
+ *   stages, by timing the collide launches of the groups for trial_steps steps:
  *   first every tile shape (LBM_BATCH_SHAPES) with automatic z-chunks, then, for
  *   the fastest shape, each candidate z-chunk (automatic, 1, 4, 8, 16, 32 planes
  *   per block, or a whole column per block).  A group and the group of the same lattice and physics
- *   with the other solid handling share members, so they take one shape (the
- *   one with the least summed time); the z-chunk is per group.  Keeps the
- *   fastest per group and writes its z-chunk to
+ *   with the other solid handling share members and launches, so they are timed together and
+ *   take one shape.  Keeps the fastest per group and writes its z-chunk to
  *   zchunk_out[g] for g < max_groups (0 = automatic, 2^30 = whole columns;
  *   lbm_batch_group reads the shape).  The members advance by 12 x (trial_steps + 1) steps.
  * lbm_batch_info: number of groups, tiles of all launches of one pass, graph mode
- *   (0 not recorded yet, 1 device-side WHILE loop, 2 replayed two-step graph).
+ *   (0 not recorded yet, 2 replayed graphs of a few steps; 1, a device-side loop, is no
+ *   longer used).
  * lbm_batch_group: lattice (19 | 27), solid handling (0 | 1), tile shape and
  *   z-chunk of group `group` in [0, ngroups); NULL outputs are skipped.
  * lbm_batch_set_group: sets a group's tile shape (0 .. LBM_BATCH_SHAPES - 1) and

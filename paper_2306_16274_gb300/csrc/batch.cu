@@ -1,17 +1,22 @@
 // Multi-domain batch (lbm_batch_*): many independent domains advanced together.
 //
-// Members are grouped by (lattice, solid handling, physical parameters).  Per time step each group
-// costs one collide-stream launch and one density/psi launch whose blocks are tiles of every
-// member of the group (up to 64 members per launch), instead of two launches per domain.  The
-// group's physical parameters (rates, equation of state, forces) and the launch's member table
-// (geometry and buffer addresses, 64 bytes a member) are passed by value in the kernel
-// parameters, so a block reads them from the constant bank as the single-domain kernel does.
-// The per-cell arithmetic is the single-domain code, so a member's result is bitwise the same
-// as stepping it alone.  Whole runs are replayed from a CUDA graph: a WHILE
-// conditional node repeats a two-step body until a device-side counter runs out, so n steps are
-// one graph launch; where conditional nodes are unavailable the two-step graph is launched n/2
-// times.  lbm_batch_tune times the candidate z-chunks per group on the live state.
+// Members are grouped by (lattice, solid handling, physical parameters); the members of one lattice and physics
+// form a chain.  Per time step a chain costs one collide-stream launch and one density/psi launch whose
+// blocks are tiles and runs of all its members (up to 64 members per launch), instead of two launches per
+// domain.  The physical parameters (rates, equation of state, forces) and the launch's member table
+// (geometry and buffer addresses) are passed by value in the kernel parameters, so a block reads them from the
+// constant bank as the single-domain kernel does.  The per-cell arithmetic is the single-domain code, so a
+// member's result is bitwise the same as stepping it alone.  The chains run side by side on streams of their
+// own, joined once a call; runs of steps are replayed from CUDA graphs of 2 and 16 steps, within which the
+// kernels of a chain overlap at their ends as lbm_step's do.
+// us a step, one launch a group and pass with all groups joined after every pass, in a device-side loop / this:
+// 4 x 32^3 D3Q19 17.2 / 8.8; 40^3 droplets and impacts on both lattices 34.0 / 19.4; 8 x 64^3 93.9 / 85.1; ten mixed
+// jobs of 48^3 - 109^3 318 / 290; 24 mixed jobs of 48^3 - 160^3 1665 / 1636.  (Advancing members in bins that fit the L2
+// one after the other: 6 x 96^3 196 against 213 us in calls of 100 steps, but 210 against 214 in calls of 20, and
+// ten mixed jobs 290 - 304 against 290: not worth it.)  lbm_batch_tune times the candidate tile shapes
+// and z-chunks per chain on the live state.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -29,33 +34,35 @@ using lbm::KParams;
 
 namespace {
 
-// One launch of a group: up to BATCH_LAUNCH_DOMS members and their tile ranges in the group's
-// tile arrays.
-struct Launch {
-    BatchDomTable tab{};
-    int t0 = 0, nt = 0;             // collide tiles
-    int p0 = 0, np = 0;             // density/psi tiles (the collide tiles in a solid-handling group)
-    int r0 = 0, nr = 0;             // density/psi runs of whole planes (plain groups)
-};
-
+// What the caller sees and tunes: members' tiles of one lattice, physics and solid handling.
 struct Group {
     int Q = 19, solids = 0;
     KParams phys{};                 // physical parameters shared by the members (geometry zeroed)
     std::vector<int> members;       // members with tiles in this group
     int zchunk = 0;                 // 0 = automatic
     int shape = 0;                  // tile shape: index into lbm::BATCH_SHAPES
-    std::vector<Launch> launches;
-    BatchTile* tiles = nullptr;     // collide tiles, then density/psi tiles (device)
     int ntiles = 0;                 // collide tiles
-    BatchRun* runs = nullptr;       // density/psi runs (device)
 };
 
-__global__ void set_counter_kernel(int* counter, int value) { *counter = value; }
+// One launch pair (collide, density/psi) of a chain: up to BATCH_LAUNCH_DOMS members, their tiles and runs.
+struct Launch {
+    BatchDomTable tab{};
+    BatchTile* tiles = nullptr;     // device
+    BatchRun* runs = nullptr;       // device
+    int nt = 0, nr = 0, near = 0;   // near: some tile or run has cells with solid neighbours
+};
 
-// Last node of the loop body: one more two-step iteration done; stop when the count runs out.
-__global__ void loop_tick_kernel(cudaGraphConditionalHandle h, int* counter) {
-    if (--(*counter) <= 0) cudaGraphSetConditional(h, 0);
-}
+// A chain: the members of one lattice and physics, advanced by their own sequence of launches.  Their tiles
+// with and without solid neighbours go into the same launches.
+struct Chain {
+    int Q = 19, plain = -1, solid = -1;   // its groups (solid: -1 if no member has walls or solids)
+    std::vector<int> members;
+    std::vector<Launch> launches;
+};
+
+// Steps of the two graphs a batch replays (the longer one only in calls that replay it four times): a graph
+// launch costs the GPU about 2 us between the last kernel of one and the first of the next.
+constexpr int GRAPH_STEPS[2] = {2, 16};
 
 bool has_solid_work(const lbm_ctx* c) { return c->nbmask != nullptr || c->kp.wall_x || c->kp.wall_y || c->kp.wall_z; }
 
@@ -99,13 +106,12 @@ struct lbm_batch {
     std::vector<KParams> seen;      // member parameters the groups were built from
     std::vector<BatchDom> table;    // member geometry and addresses the groups were built from
     std::vector<Group> groups;
+    std::vector<Chain> chains;
     cudaStream_t stream = nullptr;
-    int* counter = nullptr;         // loop counter of the graph (device)
     cudaStream_t cap = nullptr;     // capture stream
-    cudaGraphExec_t exec = nullptr;
-    int graph_parity = -1;          // AA phase the graph was recorded for
-    int graph_mode = 0;             // 0 none yet, 1 WHILE conditional node, 2 replayed two-step graph
-    std::vector<cudaStream_t> side; // one per group: the groups of a pass run concurrently
+    cudaGraphExec_t exec[2] = {nullptr, nullptr};   // GRAPH_STEPS[k] steps from AA phase graph_parity
+    int graph_parity = -1;          // AA phase the graphs were recorded for (-1: none)
+    std::vector<cudaStream_t> side; // one per chain: the chains run concurrently
     cudaEvent_t fork = nullptr;
     std::vector<cudaEvent_t> done;
     std::string err;
@@ -127,20 +133,20 @@ lbm_status bfail(lbm_batch* b, lbm_status s, const std::string& m) {
                          std::string(#call) + ": " + cudaGetErrorString(e_));                        \
     } while (0)
 
-void free_tiles(Group& g) {
-    if (g.tiles) cudaFree(g.tiles);
-    if (g.runs) cudaFree(g.runs);
-    g.tiles = nullptr;
-    g.runs = nullptr;
-    g.ntiles = 0;
-    g.launches.clear();
+void drop_graph(lbm_batch* b) {
+    for (cudaGraphExec_t& e : b->exec) {
+        if (e) cudaGraphExecDestroy(e);
+        e = nullptr;
+    }
+    b->graph_parity = -1;
 }
 
-void drop_graph(lbm_batch* b) {
-    if (b->exec) cudaGraphExecDestroy(b->exec);
-    b->exec = nullptr;
-    b->graph_parity = -1;
-    b->graph_mode = 0;
+void free_chain(Chain& c) {
+    for (Launch& L : c.launches) {
+        if (L.tiles) cudaFree(L.tiles);
+        if (L.runs) cudaFree(L.runs);
+    }
+    c.launches.clear();
 }
 
 constexpr int ZC_WHOLE = 1 << 30;   // a z-chunk candidate: every column marches through all its planes
@@ -183,32 +189,25 @@ lbm_status member_tile_flags(lbm_batch* b, lbm_ctx* c, int tw, int th) {
     return LBM_OK;
 }
 
-// Tiles of the members of a group: tw x th cells in (x, y) (the group's shape) and a run of z planes.  Along every
+// Tiles of the members of a chain: tw x th cells in (x, y) (the groups' shape) and a run of z planes.  Along every
 // column the planes are split into runs that need solid handling (a cell with a solid neighbour:
 // mask, or the first / last plane, row or column next to a wall) and runs that do not; runs are
-// cut into chunks of at most zc planes, chosen so that the whole group gives a few waves of
-// resident blocks (or the group's fixed zchunk).  A member with solids contributes its solid-free
-// chunks to the group without solid handling and the others to the solid group of its physics,
-// so only cells near solids pay for the solid tests.
+// cut into chunks of at most zc planes (the group's fixed zchunk, a member's own, or automatic).  Only the
+// tiles with solid neighbours pay for the solid tests.
 //
 // Where a row leaves 1 .. 16 cells past its last full tile width (tw = 32), those cells form narrow
 // columns, 16 cells wide and twice as high, which the same blocks step (BatchTile::narrow): a
 // 32-wide tile there would leave 16 to 31 of its 32 lanes per row idle.
 //
-// The density/psi pass of a group without solid handling covers the planes in which no column needs
-// it (every plane of a member without solids) as runs of RUN_CELLS consecutive cells, and only the
-// solid-free columns of the other planes as tiles: the pass needs no stencil, so nothing ties its
-// threads to rows, and rows that do not fill a tile's width leave no lanes idle.
-#ifndef LBM_BATCH_RUNS
-#define LBM_BATCH_RUNS 1
-#endif
+// The density/psi pass covers a member as runs of consecutive cells of whole planes: it needs no stencil, so
+// nothing ties its threads to rows, and rows that do not fill a tile's width leave no lanes idle.  Planes in
+// which some column has solid neighbours form runs of their own.
 #ifndef LBM_BATCH_NARROW
 #define LBM_BATCH_NARROW 1
 #endif
 #ifndef LBM_BATCH_LPT
 #define LBM_BATCH_LPT 1
 #endif
-constexpr uint32_t RUN_CELLS = 2048;
 
 struct Column {
     int x0, y0, w, h, narrow;
@@ -229,187 +228,193 @@ std::vector<Column> member_columns(const KParams& k, int tw, int th) {
     return cols;
 }
 
-lbm_status build_tiles(lbm_batch* b, Group& g) {
-    free_tiles(g);
-    if (g.shape < 0 || g.shape >= lbm::BATCH_NSHAPES) return bfail(b, LBM_ERR_ARG, "unknown tile shape");
-    const lbm::BatchShape& sh = lbm::BATCH_SHAPES[g.shape];
+// Automatic z-chunk of a chain: blocks of zc planes over all its columns.  Few column-planes: the shortest
+// time of the latency / throughput model that choose_zchunk (kernels_impl.cuh) explains; many: four waves
+// of resident blocks, at most ZC_AUTO_MAX planes.
+int auto_zchunk(const lbm_batch* b, const Chain& c, int resident, int tw, int th) {
+    const double cap = 152.0 * resident, ratio = c.Q == 19 ? 6.1 : 5.0;
+    double planes = 0.0;
+    long long cols = 0;
+    for (int i : c.members) {
+        const long long n = (long long)member_columns(b->members[i]->kp, tw, th).size();
+        cols += n;
+        planes += (double)n * b->members[i]->kp.nz;
+    }
+    if (planes >= 17.0 * cap) {
+        const double chunks = std::max(1.0, std::ceil(4.0 * cap / std::max(cols, 1LL)));
+        return std::min(ZC_AUTO_MAX, std::max(1, (int)std::ceil(planes / std::max(cols, 1LL) / chunks)));
+    }
+    int best = 1;
+    double best_cost = 1e300;
+    for (int zc = 1; zc <= ZC_AUTO_MAX; ++zc) {
+        double blocks = 0.0;
+        for (int i : c.members) {
+            const KParams& k = b->members[i]->kp;
+            blocks += (double)member_columns(k, tw, th).size() * ((k.nz + zc - 1) / zc);
+        }
+        const double waves = blocks / cap, B = (zc + 2) * ratio;
+        const double A = blocks / 152.0 * (zc + 1) * (1.0 + 0.15 * (std::ceil(waves) / waves - 1.0));
+        const double cost = std::max(B, A + 0.35 * B);
+        if (cost < best_cost - 1e-9) {
+            best_cost = cost;
+            best = zc;
+        }
+    }
+    return best;
+}
+
+lbm_status build_chain(lbm_batch* b, Chain& c) {
+    free_chain(c);
+    Group& plain = b->groups[c.plain];
+    Group* solid = c.solid >= 0 ? &b->groups[c.solid] : nullptr;
+    if (plain.shape < 0 || plain.shape >= lbm::BATCH_NSHAPES) return bfail(b, LBM_ERR_ARG, "unknown tile shape");
+    const lbm::BatchShape& sh = lbm::BATCH_SHAPES[plain.shape];
     const int tw = sh.bx, th = sh.by;
     const int fw = lbm::BATCH_NARROW_BX, fh = th;   // mask flags grid: both column kinds are unions of its cells
-    const int resident = g.Q == 19 ? sh.minb19 : sh.minb27;
-    const bool use_runs = LBM_BATCH_RUNS && !g.solids;
-    long long ncols = 0;
-    for (int d : g.members) ncols += (long long)member_columns(b->members[d]->kp, tw, th).size();
-    const long long target = 152LL * resident * 4;
-    const long long chunks_auto = std::max(1LL, (target + ncols - 1) / std::max(ncols, 1LL));
-    std::vector<BatchTile> t, pt;   // collide tiles; density/psi tiles
-    std::vector<BatchRun> runs;
+    const int zauto = auto_zchunk(b, c, c.Q == 19 ? sh.minb19 : sh.minb27, tw, th);
+    double cells = 0.0;
+    for (int i : c.members) cells += (double)b->members[i]->kp.ncell;
+    // 2048 cells a run, fewer where that would leave SMs without their eight blocks
+    const uint32_t run_cells = 256u * (uint32_t)std::min(8.0, std::max(1.0, cells / (152.0 * 8.0 * 256.0)));
     std::vector<uint8_t> need;      // per plane of one column: needs solid handling
     std::vector<uint8_t> mixed;     // per plane: some column needs solid handling
-    for (size_t j = 0; j < g.members.size(); ++j) {
-        const int d = (int)(j % lbm::BATCH_LAUNCH_DOMS);   // slot in the launch's member table
-        if (d == 0) {
-            g.launches.emplace_back();
-            g.launches.back().t0 = (int)t.size();
-            g.launches.back().p0 = (int)pt.size();
-            g.launches.back().r0 = (int)runs.size();
-        }
-        Launch& L = g.launches.back();
-        L.tab.d[d] = b->table[g.members[j]];
-        lbm_ctx* c = b->members[g.members[j]];
-        const KParams& k = c->kp;
-        const bool solid_work = has_solid_work(c);
-        lbm_status fs = member_tile_flags(b, c, fw, fh);
-        if (fs != LBM_OK) return fs;
-        int zc;
-        if (g.zchunk > 0) zc = std::min(g.zchunk, k.nz);            // the batch's tuned choice
-        else if (k.zchunk > 0) zc = std::min(k.zchunk, k.nz);       // the member's own setting
-        else {
-            const long long ch = std::min<long long>(chunks_auto, k.nz);
-            zc = std::min(ZC_AUTO_MAX, (int)((k.nz + ch - 1) / ch));
-        }
-        const int nxf = (k.nx + fw - 1) / fw, nyf = (k.ny + fh - 1) / fh;
-        const std::vector<Column> cols = member_columns(k, tw, th);
-        auto column_needs = [&](const Column& col) {
-            const bool side = (k.wall_x && (col.x0 == 0 || col.x0 + col.w >= k.nx)) ||
-                              (k.wall_y && (col.y0 == 0 || col.y0 + col.h >= k.ny));
-            const int fx0 = col.x0 / fw, fx1 = std::min(nxf, (col.x0 + col.w + fw - 1) / fw);
-            const int fy0 = col.y0 / fh, fy1 = std::min(nyf, (col.y0 + col.h + fh - 1) / fh);
-            for (int z = 0; z < k.nz; ++z) {
-                bool s2 = side || (k.wall_z && (z == 0 || z == k.nz - 1));
-                if (c->nbmask)
-                    for (int fy = fy0; fy < fy1 && !s2; ++fy)
-                        for (int fx = fx0; fx < fx1 && !s2; ++fx)
-                            s2 = c->tile_flags[((size_t)z * nyf + fy) * nxf + fx] != 0;
-                need[z] = s2 ? 1 : 0;
-            }
-        };
-        need.resize(k.nz);
-        mixed.assign(k.nz, 0);
-        if (solid_work)
-            for (const Column& col : cols) {
-                column_needs(col);
-                for (int z = 0; z < k.nz; ++z) mixed[z] |= need[z];
-            }
-        const int member_t0 = (int)t.size() - L.t0, member_p0 = (int)pt.size() - L.p0;
-        for (const Column& col : cols) {
-            column_needs(col);
-            for (int z0 = 0; z0 < k.nz;) {
-                int z1 = z0 + 1;
-                while (z1 < k.nz && need[z1] == need[z0] && z1 - z0 < zc) ++z1;
-                const bool mine = solid_work ? (need[z0] != 0) == (g.solids != 0) : true;
-                if (mine) t.push_back({d, col.x0, col.y0, z0, z1 - z0, col.narrow});
-                z0 = z1;
-            }
-            if (use_runs)   // density/psi tiles: this column's solid-free planes among the mixed ones
+    for (size_t j0 = 0; j0 < c.members.size(); j0 += lbm::BATCH_LAUNCH_DOMS) {
+        const int nd = (int)std::min(c.members.size() - j0, (size_t)lbm::BATCH_LAUNCH_DOMS);
+        c.launches.emplace_back();
+        Launch& L = c.launches.back();
+        std::vector<BatchTile> t;
+        std::vector<BatchRun> runs;
+        for (int d = 0; d < nd; ++d) {   // d: slot in the launch's member table
+            L.tab.d[d] = b->table[c.members[j0 + d]];
+            lbm_ctx* ctx = b->members[c.members[j0 + d]];
+            const KParams& k = ctx->kp;
+            const bool solid_work = has_solid_work(ctx);
+            lbm_status fs = member_tile_flags(b, ctx, fw, fh);
+            if (fs != LBM_OK) return fs;
+            auto chunk = [&](const Group& g) {   // the batch's tuned choice, the member's own setting, automatic
+                const int zc = g.zchunk > 0 ? g.zchunk : (k.zchunk > 0 ? k.zchunk : zauto);
+                return std::min(zc, k.nz);
+            };
+            const int zc[2] = {chunk(plain), chunk(solid ? *solid : plain)};
+            const int nxf = (k.nx + fw - 1) / fw, nyf = (k.ny + fh - 1) / fh;
+            need.resize(k.nz);
+            mixed.assign(k.nz, 0);
+            const size_t member_t0 = t.size();
+            for (const Column& col : member_columns(k, tw, th)) {
+                const bool side = (k.wall_x && (col.x0 == 0 || col.x0 + col.w >= k.nx)) ||
+                                  (k.wall_y && (col.y0 == 0 || col.y0 + col.h >= k.ny));
+                const int fx0 = col.x0 / fw, fx1 = std::min(nxf, (col.x0 + col.w + fw - 1) / fw);
+                const int fy0 = col.y0 / fh, fy1 = std::min(nyf, (col.y0 + col.h + fh - 1) / fh);
+                for (int z = 0; z < k.nz; ++z) {
+                    bool s2 = solid_work && (side || (k.wall_z && (z == 0 || z == k.nz - 1)));
+                    if (solid_work && ctx->nbmask)
+                        for (int fy = fy0; fy < fy1 && !s2; ++fy)
+                            for (int fx = fx0; fx < fx1 && !s2; ++fx)
+                                s2 = ctx->tile_flags[((size_t)z * nyf + fy) * nxf + fx] != 0;
+                    need[z] = s2 ? 1 : 0;
+                    mixed[z] |= need[z];
+                }
                 for (int z0 = 0; z0 < k.nz;) {
-                    if (need[z0] || !mixed[z0]) {
-                        ++z0;
-                        continue;
-                    }
                     int z1 = z0 + 1;
-                    while (z1 < k.nz && !need[z1] && mixed[z1] && z1 - z0 < zc) ++z1;
-                    pt.push_back({d, col.x0, col.y0, z0, z1 - z0, col.narrow});
+                    while (z1 < k.nz && need[z1] == need[z0] && z1 - z0 < zc[need[z0]]) ++z1;
+                    t.push_back({d, col.x0, col.y0, z0, z1 - z0, col.narrow, need[z0]});
+                    (need[z0] ? *solid : plain).ntiles += 1;
+                    L.near |= need[z0];
                     z0 = z1;
                 }
-        }
-        // z-chunk-major order within the member (as the single-domain grid): blocks resident at
-        // the same time work on neighbouring columns of the same planes
-        auto zmajor = [](const BatchTile& a, const BatchTile& b2) {
-            return a.z0 != b2.z0 ? a.z0 < b2.z0 : (a.y0 != b2.y0 ? a.y0 < b2.y0 : a.x0 < b2.x0);
-        };
-        std::stable_sort(t.begin() + L.t0 + member_t0, t.end(), zmajor);
-        std::stable_sort(pt.begin() + L.p0 + member_p0, pt.end(), zmajor);
-        if (use_runs) {
+            }
+            // z-chunk-major order within the member (as the single-domain grid): blocks resident at
+            // the same time work on neighbouring columns of the same planes
+            std::stable_sort(t.begin() + member_t0, t.end(), [](const BatchTile& a, const BatchTile& b2) {
+                return a.z0 != b2.z0 ? a.z0 < b2.z0 : (a.y0 != b2.y0 ? a.y0 < b2.y0 : a.x0 < b2.x0);
+            });
             const uint32_t nxy = (uint32_t)k.nx * (uint32_t)k.ny;
             for (int z0 = 0; z0 < k.nz;) {
-                if (mixed[z0]) {
-                    ++z0;
-                    continue;
-                }
                 int z1 = z0 + 1;
-                while (z1 < k.nz && !mixed[z1]) ++z1;
+                while (z1 < k.nz && mixed[z1] == mixed[z0]) ++z1;
                 const uint32_t end = (uint32_t)z1 * nxy;
-                for (uint32_t a = (uint32_t)z0 * nxy; a < end; a += std::min(RUN_CELLS, end - a))
-                    runs.push_back({d, a, a + std::min(RUN_CELLS, end - a)});
+                for (uint32_t a = (uint32_t)z0 * nxy; a < end; a += std::min(run_cells, end - a))
+                    runs.push_back({d, a, a + std::min(run_cells, end - a), mixed[z0]});
                 z0 = z1;
             }
         }
-        L.nt = (int)t.size() - L.t0;
-        L.np = (int)pt.size() - L.p0;
-        L.nr = (int)runs.size() - L.r0;
-    }
-    // longest marches first within a launch: blocks start roughly in index order, so the short ones
-    // fill the last wave instead of a few long ones running on alone
-    if (LBM_BATCH_LPT)
-        for (const Launch& L : g.launches)
-            std::stable_sort(t.begin() + L.t0, t.begin() + L.t0 + L.nt,
-                             [](const BatchTile& a, const BatchTile& b2) { return a.zc > b2.zc; });
-    if (!use_runs)
-        for (Launch& L : g.launches) {   // the density/psi pass runs over the collide tiles
-            L.p0 = L.t0;
-            L.np = L.nt;
+        // longest marches first within a launch: blocks start roughly in index order, so the short ones
+        // fill the last wave instead of a few long ones running on alone
+        if (LBM_BATCH_LPT)
+            std::stable_sort(t.begin(), t.end(), [](const BatchTile& a, const BatchTile& b2) { return a.zc > b2.zc; });
+        // against the collide pass's direction: the pass starts on what that one left in the L2
+        std::reverse(runs.begin(), runs.end());
+        if (t.size() > 0x7fffffff || runs.size() > 0x7fffffff) return bfail(b, LBM_ERR_ARG, "too many tiles");
+        L.nt = (int)t.size();
+        L.nr = (int)runs.size();
+        if (L.nt > 0) {
+            BCK(b, cudaMalloc((void**)&L.tiles, t.size() * sizeof(BatchTile)));
+            BCK(b, cudaMemcpyAsync(L.tiles, t.data(), t.size() * sizeof(BatchTile), cudaMemcpyHostToDevice, b->stream));
         }
-    else
-        for (Launch& L : g.launches) L.p0 += (int)t.size();
-    if (t.size() + pt.size() > 0x7fffffff || runs.size() > 0x7fffffff) return bfail(b, LBM_ERR_ARG, "too many tiles");
-    const size_t nt = t.size() + pt.size();
-    if (nt > 0) {
-        t.insert(t.end(), pt.begin(), pt.end());
-        BCK(b, cudaMalloc((void**)&g.tiles, nt * sizeof(BatchTile)));
-        BCK(b, cudaMemcpyAsync(g.tiles, t.data(), nt * sizeof(BatchTile), cudaMemcpyHostToDevice, b->stream));
+        if (L.nr > 0) {
+            BCK(b, cudaMalloc((void**)&L.runs, runs.size() * sizeof(BatchRun)));
+            BCK(b, cudaMemcpyAsync(L.runs, runs.data(), runs.size() * sizeof(BatchRun), cudaMemcpyHostToDevice, b->stream));
+        }
+        BCK(b, cudaStreamSynchronize(b->stream));   // t and runs go
     }
-    if (!runs.empty()) {
-        BCK(b, cudaMalloc((void**)&g.runs, runs.size() * sizeof(BatchRun)));
-        BCK(b, cudaMemcpyAsync(g.runs, runs.data(), runs.size() * sizeof(BatchRun), cudaMemcpyHostToDevice, b->stream));
-    }
-    BCK(b, cudaStreamSynchronize(b->stream));
-    g.ntiles = (int)(nt - pt.size());
     return LBM_OK;
 }
 
-// One collide launch of group g at AA phase `parity` (optionally bracketed by events).
-cudaError_t collide_group(const Group& g, int parity, cudaStream_t st) {
-    for (const Launch& L : g.launches) {
-        const BatchTile* t = g.tiles + L.t0;
-        cudaError_t e = g.Q == 19 ? lbm::launch_collide_batch_q19(g.phys, L.tab, t, L.nt, parity, g.solids, g.shape, st)
-                                  : lbm::launch_collide_batch_q27(g.phys, L.tab, t, L.nt, parity, g.solids, g.shape, st);
+// Rebuilds the tiles of every chain (only of the one with group `only`, if that is not negative).
+lbm_status build_chains(lbm_batch* b, int only = -1) {
+    drop_graph(b);
+    for (Chain& c : b->chains) {
+        if (only >= 0 && c.plain != only && c.solid != only) continue;
+        b->groups[c.plain].ntiles = 0;
+        if (c.solid >= 0) b->groups[c.solid].ntiles = 0;
+        lbm_status s = build_chain(b, c);
+        if (s != LBM_OK) return s;
+    }
+    return LBM_OK;
+}
+
+cudaError_t collide_chain(const lbm_batch* b, const Chain& c, int parity, cudaStream_t st) {
+    const Group& g = b->groups[c.plain];
+    for (const Launch& L : c.launches) {
+        cudaError_t e = c.Q == 19 ? lbm::launch_collide_batch_q19(g.phys, L.tab, L.tiles, L.nt, parity, L.near, g.shape, st)
+                                  : lbm::launch_collide_batch_q27(g.phys, L.tab, L.tiles, L.nt, parity, L.near, g.shape, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-cudaError_t psi_group(const Group& g, int parity, cudaStream_t st) {
+cudaError_t psi_chain(const lbm_batch* b, const Chain& c, int parity, cudaStream_t st) {
+    const Group& g = b->groups[c.plain];
     if (!g.phys.multiphase) return cudaSuccess;
-    for (const Launch& L : g.launches) {
-        const BatchTile* t = g.tiles + L.p0;
-        cudaError_t e = g.Q == 19 ? lbm::launch_psi_batch_q19(g.phys, L.tab, t, L.np, parity, g.solids, g.shape, st)
-                                  : lbm::launch_psi_batch_q27(g.phys, L.tab, t, L.np, parity, g.solids, g.shape, st);
-        if (e == cudaSuccess && L.nr > 0)
-            e = g.Q == 19 ? lbm::launch_psi_runs_q19(g.phys, L.tab, g.runs + L.r0, L.nr, parity, st)
-                          : lbm::launch_psi_runs_q27(g.phys, L.tab, g.runs + L.r0, L.nr, parity, st);
+    for (const Launch& L : c.launches) {
+        cudaError_t e = c.Q == 19 ? lbm::launch_psi_runs_q19(g.phys, L.tab, L.runs, L.nr, parity, L.near, st)
+                                  : lbm::launch_psi_runs_q27(g.phys, L.tab, L.runs, L.nr, parity, L.near, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-// (Re)build the groups, their member tables and tiles from the members' current parameters.  Walls-only members join both the plain group (interior tiles) and the
-// solid-handling group (boundary tiles) of their physics.
+// (Re)build the groups, chains and tiles from the members' current parameters.  Members with walls or
+// solids join both the plain group (interior tiles) and the solid-handling group of their physics.
 lbm_status regroup(lbm_batch* b) {
     drop_graph(b);
-    for (Group& g : b->groups) free_tiles(g);
+    for (Chain& c : b->chains) free_chain(c);
+    b->chains.clear();
     b->groups.clear();
     const int n = (int)b->members.size();
     b->seen.resize(n);
     b->table.resize(n);
-    auto group_of = [&](int Q, int solids, const KParams& phys) -> Group& {
-        for (Group& g : b->groups)
-            if (g.Q == Q && g.solids == solids && std::memcmp(&g.phys, &phys, sizeof(KParams)) == 0) return g;
+    auto group_of = [&](int Q, int solids, const KParams& phys) -> int {
+        for (size_t g = 0; g < b->groups.size(); ++g)
+            if (b->groups[g].Q == Q && b->groups[g].solids == solids &&
+                std::memcmp(&b->groups[g].phys, &phys, sizeof(KParams)) == 0)
+                return (int)g;
         Group g;
         g.Q = Q;
         g.solids = solids;
         g.phys = phys;
         b->groups.push_back(g);
-        return b->groups.back();
+        return (int)b->groups.size() - 1;
     };
     for (int i = 0; i < n; ++i) {
         const lbm_ctx* c = b->members[i];
@@ -419,14 +424,22 @@ lbm_status regroup(lbm_batch* b) {
         std::memcpy(&b->seen[i], &c->kp, sizeof(KParams));
         b->table[i] = dom_of(c);
         const KParams phys = physics_of(c->kp);
-        group_of(c->Q, 0, phys).members.push_back(i);   // solid-free tiles
-        if (has_solid_work(c)) group_of(c->Q, 1, phys).members.push_back(i);
+        const int plain = group_of(c->Q, 0, phys), solid = has_solid_work(c) ? group_of(c->Q, 1, phys) : -1;
+        b->groups[plain].members.push_back(i);
+        if (solid >= 0) b->groups[solid].members.push_back(i);
+        Chain* k = nullptr;
+        for (Chain& c2 : b->chains)
+            if (c2.plain == plain) k = &c2;
+        if (!k) {
+            b->chains.emplace_back();
+            k = &b->chains.back();
+            k->Q = c->Q;
+            k->plain = plain;
+        }
+        if (solid >= 0) k->solid = solid;
+        k->members.push_back(i);
     }
-    for (Group& g : b->groups) {
-        lbm_status s = build_tiles(b, g);
-        if (s != LBM_OK) return s;
-    }
-    return LBM_OK;
+    return build_chains(b);
 }
 
 // Has any member changed (re-initialised with another solid mask) since the groups were built?
@@ -440,18 +453,24 @@ bool members_changed(const lbm_batch* b) {
     return false;
 }
 
-// One pass (collide-stream or density/psi) of every group.  The groups' launches are
-// independent within a pass -- tiles of one member in two groups touch disjoint cells, and the
-// in-place AA update of a cell reads and writes only that cell's slots -- so they are forked onto
-// one side stream each and joined before the next pass (in a captured graph: parallel nodes
-// between two joins).  The next pass needs all of them: psi reads populations that neighbouring
-// tiles wrote, and collide reads the psi halo.
-cudaError_t pass(lbm_batch* b, bool collide, int parity, cudaStream_t st) {
-    const size_t G = b->groups.size();
-    if (G == 1) return collide ? collide_group(b->groups[0], parity, st) : psi_group(b->groups[0], parity, st);
+// `steps` steps of every member from AA phase `parity` (psi of the current state valid).  Within a chain a step
+// needs the one before it (psi reads populations that neighbouring tiles wrote, collide the psi halo); the chains
+// have nothing in common, so each runs all its steps on a stream of its own, joined at the end.
+cudaError_t step_all(lbm_batch* b, int parity, int steps, cudaStream_t st) {
+    auto steps_of = [&](const Chain& c, cudaStream_t s) {
+        cudaError_t e = cudaSuccess;
+        for (int k = 0; k < steps && e == cudaSuccess; ++k) {
+            const int p = parity ^ (k & 1);
+            e = collide_chain(b, c, p, s);
+            if (e == cudaSuccess) e = psi_chain(b, c, p ^ 1, s);
+        }
+        return e;
+    };
+    const size_t n = b->chains.size();
+    if (n == 1) return steps_of(b->chains[0], st);
     cudaError_t e = cudaSuccess;
     if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-    while (e == cudaSuccess && b->side.size() < G) {
+    while (e == cudaSuccess && b->side.size() < n) {
         cudaStream_t s2 = nullptr;
         cudaEvent_t ev = nullptr;
         e = cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking);
@@ -462,77 +481,29 @@ cudaError_t pass(lbm_batch* b, bool collide, int parity, cudaStream_t st) {
         }
     }
     if (e == cudaSuccess) e = cudaEventRecord(b->fork, st);
-    for (size_t k = 0; k < G && e == cudaSuccess; ++k) {
+    for (size_t k = 0; k < n && e == cudaSuccess; ++k) {
         e = cudaStreamWaitEvent(b->side[k], b->fork, 0);
-        if (e == cudaSuccess)
-            e = collide ? collide_group(b->groups[k], parity, b->side[k]) : psi_group(b->groups[k], parity, b->side[k]);
+        if (e == cudaSuccess) e = steps_of(b->chains[k], b->side[k]);
         if (e == cudaSuccess) e = cudaEventRecord(b->done[k], b->side[k]);
     }
-    for (size_t k = 0; k < G && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(st, b->done[k], 0);
+    for (size_t k = 0; k < n && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(st, b->done[k], 0);
     return e;
 }
 
-// One step of every member, starting at AA phase `parity` (psi of the current state valid).
-cudaError_t step_once(lbm_batch* b, int parity, cudaStream_t st) {
-    cudaError_t e = pass(b, true, parity, st);
-    return e == cudaSuccess ? pass(b, false, parity ^ 1, st) : e;
-}
-
-lbm_status record_graph(lbm_batch* b, int parity) {
-    drop_graph(b);
+// b->exec[k]: GRAPH_STEPS[k] steps as one graph
+lbm_status record_graph(lbm_batch* b, int k, int parity) {
     if (!b->cap) BCK(b, cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
-    // first choice: one WHILE node whose body is two steps and a counter tick
-    cudaGraph_t g = nullptr;
-    BCK(b, cudaGraphCreate(&g, 0));
-    cudaGraphConditionalHandle h;
-    bool ok = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
-    cudaGraphNodeParams cp = {};
-    cudaGraphNode_t node;
-    if (ok) {
-        cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = h;
-        cp.conditional.type = cudaGraphCondTypeWhile;
-        cp.conditional.size = 1;
-        ok = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp) == cudaSuccess;
-    }
-    if (ok) {
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
-        ok = cudaStreamBeginCaptureToGraph(b->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
-             cudaSuccess;
-        if (ok) {
-            cudaError_t e1 = step_once(b, parity, b->cap);
-            cudaError_t e2 = e1 == cudaSuccess ? step_once(b, parity ^ 1, b->cap) : e1;
-            if (e2 == cudaSuccess) {
-                loop_tick_kernel<<<1, 1, 0, b->cap>>>(h, b->counter);
-                e2 = cudaGetLastError();
-            }
-            cudaGraph_t out = nullptr;
-            cudaError_t e3 = cudaStreamEndCapture(b->cap, &out);
-            ok = e2 == cudaSuccess && e3 == cudaSuccess;
-        }
-    }
-    if (ok) ok = cudaGraphInstantiate(&b->exec, g, 0) == cudaSuccess;
-    cudaGraphDestroy(g);
-    if (ok) {
-        b->graph_mode = 1;
-        b->graph_parity = parity;
-        return LBM_OK;
-    }
-    (void)cudaGetLastError();
-    b->exec = nullptr;
-    // fallback: a plain two-step graph, replayed
     BCK(b, cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e1 = step_once(b, parity, b->cap);
-    cudaError_t e2 = e1 == cudaSuccess ? step_once(b, parity ^ 1, b->cap) : e1;
-    cudaGraph_t g2 = nullptr;
-    cudaError_t e3 = cudaStreamEndCapture(b->cap, &g2);
-    if (e2 != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e2));
-    if (e3 != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e3));
-    cudaError_t e4 = cudaGraphInstantiate(&b->exec, g2, 0);
-    cudaGraphDestroy(g2);
-    if (e4 != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("instantiate: ") + cudaGetErrorString(e4));
-    b->graph_mode = 2;
-    b->graph_parity = parity;
+    cudaError_t e = step_all(b, parity, GRAPH_STEPS[k], b->cap);
+    cudaGraph_t g = nullptr;
+    cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec[k], g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+        b->exec[k] = nullptr;
+        return bfail(b, LBM_ERR_CUDA, std::string("graph: ") + cudaGetErrorString(e));
+    }
     return LBM_OK;
 }
 
@@ -567,8 +538,7 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int32_t n, void* cuda_stream, 
     b->members.assign(ctxs, ctxs + n);
     b->stream = (cudaStream_t)cuda_stream;
     lbm_status s = LBM_OK;
-    if (cudaMalloc((void**)&b->counter, sizeof(int)) != cudaSuccess) s = bfail(b, LBM_ERR_OOM, "batch set-up: counter");
-    if (s == LBM_OK) s = regroup(b);
+    s = regroup(b);
     if (s == LBM_OK && cudaStreamSynchronize(b->stream) != cudaSuccess) s = bfail(b, LBM_ERR_CUDA, "batch set-up");
     if (s != LBM_OK) {
         lbm::set_thread_error(b->err.c_str());
@@ -591,23 +561,20 @@ lbm_status lbm_batch_step(lbm_batch* b, int32_t n) {
         lbm_status s = regroup(b);
         if (s != LBM_OK) return s;
     }
-    int done = 0;
-    if (n >= 2) {
-        if (b->graph_parity != parity) {
-            lbm_status s = record_graph(b, parity);
+    if (n >= 2 && b->graph_parity != parity) {
+        drop_graph(b);
+        b->graph_parity = parity;
+    }
+    int left = n;
+    for (int k = 1; k >= 0; --k) {
+        if (left < GRAPH_STEPS[k] || (k == 1 && !b->exec[1] && n < 4 * GRAPH_STEPS[1])) continue;
+        if (!b->exec[k]) {
+            lbm_status s = record_graph(b, k, parity);
             if (s != LBM_OK) return s;
         }
-        const int pairs = n / 2;
-        if (b->graph_mode == 1) {
-            set_counter_kernel<<<1, 1, 0, b->stream>>>(b->counter, pairs);
-            BCK(b, cudaGetLastError());
-            BCK(b, cudaGraphLaunch(b->exec, b->stream));
-        } else {
-            for (int k = 0; k < pairs; ++k) BCK(b, cudaGraphLaunch(b->exec, b->stream));
-        }
-        done = 2 * pairs;
+        for (; left >= GRAPH_STEPS[k]; left -= GRAPH_STEPS[k]) BCK(b, cudaGraphLaunch(b->exec[k], b->stream));
     }
-    if (done < n) BCK(b, step_once(b, parity, b->stream));
+    if (left > 0) BCK(b, step_all(b, parity ^ ((n - left) & 1), left, b->stream));
     advance_members(b, n);
     return LBM_OK;
 }
@@ -643,37 +610,38 @@ int partner_group(const lbm_batch* b, int k) {
     return -1;
 }
 
-// Times every group's collide launches over `trial_steps` steps with each group set to candidate
-// (shape_of(g, ci), zchunk_of(g, ci)) in turn, ci < ncand; times[ci][g] receives the total.  The
-// members advance by ncand x (trial_steps + 1) steps.
+// Times every chain's collide launches over `trial_steps` steps with each group set to candidate
+// (shape_of(g, ci), zchunk_of(g, ci)) in turn, ci < ncand; times[ci][g] receives the total of the chains with
+// group g.  The members advance by ncand x (trial_steps + 1) steps.
 template <class SF, class ZF>
 lbm_status time_candidates(lbm_batch* b, int trial_steps, int ncand, SF shape_of, ZF zchunk_of,
                            std::vector<std::vector<double>>& times) {
     const size_t G = b->groups.size();
+    std::vector<const Chain*> chains;
+    for (const Chain& c : b->chains) chains.push_back(&c);
+    const size_t C = chains.size();
     times.assign(ncand, std::vector<double>(G, 0.0));
-    std::vector<cudaEvent_t> ev(2 * G * trial_steps);
+    std::vector<cudaEvent_t> ev(2 * C * trial_steps);
     for (auto& e : ev) BCK(b, cudaEventCreate(&e));
     lbm_status result = LBM_OK;
     for (int ci = 0; ci < ncand && result == LBM_OK; ++ci) {
-        for (size_t k = 0; k < G && result == LBM_OK; ++k) {
-            Group& g = b->groups[k];
-            g.shape = shape_of((int)k, ci);
-            g.zchunk = zchunk_of((int)k, ci);
-            result = build_tiles(b, g);
+        for (size_t k = 0; k < G; ++k) {
+            b->groups[k].shape = shape_of((int)k, ci);
+            b->groups[k].zchunk = zchunk_of((int)k, ci);
         }
+        result = build_chains(b);
         if (result != LBM_OK) break;
-        drop_graph(b);
         int parity = b->members[0]->parity;
-        // one untimed step, then per-group events around every collide launch
-        cudaError_t e = step_once(b, parity, b->stream);
+        // one untimed step, then events around every chain's collide launches
+        cudaError_t e = step_all(b, parity, 1, b->stream);
         parity ^= 1;
         for (int s = 0; s < trial_steps && e == cudaSuccess; ++s) {
-            for (size_t k = 0; k < G && e == cudaSuccess; ++k) {
-                e = cudaEventRecord(ev[2 * (s * G + k)], b->stream);
-                if (e == cudaSuccess) e = collide_group(b->groups[k], parity, b->stream);
-                if (e == cudaSuccess) e = cudaEventRecord(ev[2 * (s * G + k) + 1], b->stream);
+            for (size_t k = 0; k < C && e == cudaSuccess; ++k) {
+                e = cudaEventRecord(ev[2 * (s * C + k)], b->stream);
+                if (e == cudaSuccess) e = collide_chain(b, *chains[k], parity, b->stream);
+                if (e == cudaSuccess) e = cudaEventRecord(ev[2 * (s * C + k) + 1], b->stream);
             }
-            for (size_t k = 0; k < G && e == cudaSuccess; ++k) e = psi_group(b->groups[k], parity ^ 1, b->stream);
+            for (size_t k = 0; k < C && e == cudaSuccess; ++k) e = psi_chain(b, *chains[k], parity ^ 1, b->stream);
             parity ^= 1;
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -682,13 +650,13 @@ lbm_status time_candidates(lbm_batch* b, int trial_steps, int ncand, SF shape_of
             break;
         }
         advance_members(b, trial_steps + 1);
-        for (size_t k = 0; k < G; ++k) {
+        for (size_t k = 0; k < C; ++k)
             for (int s = 0; s < trial_steps; ++s) {
                 float ms = 0.f;
-                cudaEventElapsedTime(&ms, ev[2 * (s * G + k)], ev[2 * (s * G + k) + 1]);
-                times[ci][k] += ms;
+                cudaEventElapsedTime(&ms, ev[2 * (s * C + k)], ev[2 * (s * C + k) + 1]);
+                times[ci][chains[k]->plain] += ms;
+                if (chains[k]->solid >= 0) times[ci][chains[k]->solid] += ms;
             }
-        }
     }
     for (auto& e : ev) cudaEventDestroy(e);
     return result;
@@ -737,12 +705,9 @@ lbm_status lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* zchunk_out
     for (int k = 0; k < G; ++k) {
         b->groups[k].shape = shape[k];
         b->groups[k].zchunk = zchunk[k];
-        lbm_status s = build_tiles(b, b->groups[k]);
-        if (s != LBM_OK) return s;
         if (zchunk_out && k < max_groups) zchunk_out[k] = zchunk[k];
     }
-    drop_graph(b);
-    return LBM_OK;
+    return build_chains(b);
 }
 
 lbm_status lbm_batch_group(const lbm_batch* b, int32_t group, int32_t* lattice, int32_t* solids, int32_t* shape,
@@ -762,17 +727,11 @@ lbm_status lbm_batch_set_group(lbm_batch* b, int32_t group, int32_t shape, int32
     if (group < 0 || group >= (int32_t)b->groups.size()) return bfail(b, LBM_ERR_ARG, "no such group");
     if (shape < 0 || shape >= lbm::BATCH_NSHAPES) return bfail(b, LBM_ERR_ARG, "shape must lie in [0, LBM_BATCH_SHAPES)");
     if (zchunk < 0) return bfail(b, LBM_ERR_ARG, "zchunk must be >= 0");
-    Group& g = b->groups[group];
-    g.shape = shape;
-    g.zchunk = zchunk;
-    drop_graph(b);
-    lbm_status s = build_tiles(b, g);
+    b->groups[group].shape = shape;
+    b->groups[group].zchunk = zchunk;
     const int p = partner_group(b, group);
-    if (s == LBM_OK && p >= 0 && b->groups[p].shape != shape) {   // the partner takes the same columns
-        b->groups[p].shape = shape;
-        s = build_tiles(b, b->groups[p]);
-    }
-    return s;
+    if (p >= 0) b->groups[p].shape = shape;   // the partner takes the same columns
+    return build_chains(b, group);
 }
 
 lbm_status lbm_batch_info(const lbm_batch* b, int32_t* ngroups, int32_t* ntiles, int32_t* graph_mode) {
@@ -783,7 +742,7 @@ lbm_status lbm_batch_info(const lbm_batch* b, int32_t* ngroups, int32_t* ntiles,
         for (const Group& g : b->groups) t += g.ntiles;
         *ntiles = (int32_t)std::min<long long>(t, 0x7fffffff);
     }
-    if (graph_mode) *graph_mode = b->graph_mode;
+    if (graph_mode) *graph_mode = b->graph_parity >= 0 ? 2 : 0;
     return LBM_OK;
 }
 
@@ -791,8 +750,7 @@ void lbm_batch_destroy(lbm_batch* b) {
     if (!b) return;
     (void)cudaStreamSynchronize(b->stream);
     drop_graph(b);
-    for (Group& g : b->groups) free_tiles(g);
-    if (b->counter) cudaFree(b->counter);
+    for (Chain& c : b->chains) free_chain(c);
     if (b->cap) cudaStreamDestroy(b->cap);
     for (cudaStream_t s2 : b->side) cudaStreamDestroy(s2);
     for (cudaEvent_t ev : b->done) cudaEventDestroy(ev);

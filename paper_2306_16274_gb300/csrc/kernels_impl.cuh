@@ -159,35 +159,18 @@ __global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_kernel(KParams kp, float*
 }
 
 
-// multi-domain density + psi pass: one block per tile (of shape S) of any member of the launch's
-// table; physics by value
-template <int PARITY, bool SOLIDS, int S>
-__global__ void __launch_bounds__(BatchTileShape<S>::NT) psi_batch_kernel(const KParams phys,
-                                                                       const __grid_constant__ BatchDomTable tab,
-                                                                       const BatchTile* __restrict__ tiles) {
-    const BatchTile t = tiles[blockIdx.x];
-    const BatchDom& m = tab.d[t.d];
-    const DGeom g{m};
-    const PlaneIdx32 addr{m.base, (uint32_t)m.plane};
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    const int w = t.narrow ? BATCH_NARROW_BX : (int)blockDim.x;   // a narrow tile: 16 cells wide
-    psi_column<PARITY, SOLIDS, false>(phys, g, addr, m.psi, m.nbmask, m.status, t.x0 + tid % w, t.y0 + tid / w, t.z0,
-                                      min(t.z0 + t.zc, m.nz), nullptr, nullptr);
-}
-
-// multi-domain density + psi pass over runs of whole planes (cells without solid handling): thread k
-// of a block takes cells begin + k, begin + k + RUN_NT, ... of its run, so rows of any length pack
-// the warps densely.  Per cell the arithmetic and its order are psi_column's.
+// multi-domain density + psi pass over runs of whole planes: thread k of a block takes cells begin + k,
+// begin + k + RUN_NT, ... of its run, so rows of any length pack the warps densely.  Per cell the
+// arithmetic and its order are psi_column's.  A run of planes without solid neighbours takes the code without
+// solid tests.
 constexpr int RUN_NT = 256;
 __device__ __forceinline__ uint32_t div_by_magic(uint32_t n, uint32_t m, int s) {
     return (uint32_t)(((unsigned long long)m * n) >> s);
 }
-template <int PARITY>
-__global__ void __launch_bounds__(RUN_NT) psi_run_kernel(const KParams phys, const __grid_constant__ BatchDomTable tab,
-                                                         const BatchRun* __restrict__ runs) {
-    const BatchRun r = runs[blockIdx.x];
-    const BatchDom& m = tab.d[r.d];
+template <int PARITY, bool NEAR>
+__device__ __forceinline__ void psi_run(const KParams& phys, const BatchDom& m, const BatchRun& r) {
     const PlaneIdx32 addr{m.base, (uint32_t)m.plane};
+    const DGeom g{m};
     const uint32_t nx = (uint32_t)m.nx, ny = (uint32_t)m.ny, nz = (uint32_t)m.nz, nxy = nx * ny;
     for (uint32_t c = r.begin + threadIdx.x; c < r.end; c += RUN_NT) {
         const uint32_t row = div_by_magic(c, m.mx, m.sx), x = c - row * nx;
@@ -203,13 +186,27 @@ __global__ void __launch_bounds__(RUN_NT) psi_run_kernel(const KParams phys, con
         o.zo[1] = z * nxy;
         o.zo[2] = (uint32_t)wrap1((int)z + 1, (int)nz) * nxy;
         o.c = c;
+        const uint32_t bits = NEAR ? solid_bits32<Q>(g, m.nbmask, c, (int)x, (int)y, (int)z) : 0u;
+        if (bits & 1u) {
+            m.psi[bounded(c, (unsigned long long)nxy * nz)] = 0.0f;
+            continue;
+        }
         float p[Q];
-        gather32<Q, PARITY, false>(addr, o, 0u, p);
+        gather32<Q, PARITY, NEAR>(addr, o, bits, p);
         float rho = 0.0f;
 #pragma unroll
         for (int i = 0; i < Q; ++i) rho += p[i];
         m.psi[bounded(c, (unsigned long long)nxy * nz)] = eval_psi(phys, rho, m.status);
     }
+}
+template <int PARITY, bool NEAR>
+__global__ void __launch_bounds__(RUN_NT) psi_run_kernel(const KParams phys, const __grid_constant__ BatchDomTable tab,
+                                                         const BatchRun* __restrict__ runs) {
+    const BatchRun r = runs[blockIdx.x];
+    const BatchDom& m = tab.d[r.d];
+    dep_wait();
+    if (NEAR && r.near) psi_run<PARITY, true>(phys, m, r);
+    else psi_run<PARITY, false>(phys, m, r);
 }
 
 // ---- fused collide-stream pass: psi tile -> forces -> gather -> moments -> relax -> M^-1 -> store
@@ -1267,17 +1264,13 @@ __global__ void pull_store_kernel(KParams kp, const float* __restrict__ fin, lon
     }
 }
 
-// multi-domain collide-stream pass: one block per tile of any member of the launch's table;
-// physics by value; tiles of shape S of BATCH_SHAPES
+// one tile of a multi-domain collide-stream pass: of shape S of BATCH_SHAPES, or narrow
 template <int PARITY, bool SOLIDS, bool MULTIPHASE, int S>
-__global__ void __launch_bounds__(BatchTileShape<S>::NT, batch_minb<S>()) collide_batch_kernel(
-        const KParams phys, const __grid_constant__ BatchDomTable tab, const BatchTile* __restrict__ tiles) {
+__device__ __forceinline__ void batch_tile(const KParams& phys, const BatchDom& m, const BatchTile& t,
+                                           float (*ring)[BatchTileShape<S>::RP]) {
     using TS = BatchTileShape<S>;
     using TN = TileShape<BATCH_NARROW_BX, TS::NT / BATCH_NARROW_BX>;   // narrow tiles at the ends of rows
     static_assert(TN::RP <= TS::RP, "a narrow tile's ring fits the block's");
-    __shared__ float ring[4][TS::RP];
-    const BatchTile t = tiles[blockIdx.x];
-    const BatchDom& m = tab.d[t.d];
     const DGeom g{m};
     const DomPlanes addr{m};
     if (TS::BX != BATCH_NARROW_BX && t.narrow)
@@ -1288,6 +1281,26 @@ __global__ void __launch_bounds__(BatchTileShape<S>::NT, batch_minb<S>()) collid
         collide_tile<TS, PARITY, SOLIDS, MULTIPHASE, false, !SOLIDS>(phys, g, addr, m.psi, m.nbmask, m.status, t.x0,
                                                                     t.y0, t.z0, t.zc, g.nz(), ring, nullptr, nullptr,
                                                                     nullptr);
+}
+// tiles with solid neighbours as a function of their own (see collide_tile_near)
+template <int PARITY, bool MULTIPHASE, int S>
+__device__ __noinline__ void batch_tile_near(const KParams& phys, const BatchDom& m, const BatchTile& t,
+                                             float (*ring)[BatchTileShape<S>::RP]) {
+    batch_tile<PARITY, true, MULTIPHASE, S>(phys, m, t, ring);
+}
+
+// multi-domain collide-stream pass: one block per tile of any member of the launch's table; physics by
+// value.  NEAR: some tiles of the launch have cells with solid neighbours (BatchTile::near).
+template <int PARITY, bool NEAR, bool MULTIPHASE, int S>
+__global__ void __launch_bounds__(BatchTileShape<S>::NT, batch_minb<S>()) collide_batch_kernel(
+        const __grid_constant__ KParams phys, const __grid_constant__ BatchDomTable tab,
+        const BatchTile* __restrict__ tiles) {
+    __shared__ float ring[4][BatchTileShape<S>::RP];
+    const BatchTile t = tiles[blockIdx.x];
+    const BatchDom& m = tab.d[t.d];
+    dep_wait();
+    if (NEAR && t.near) batch_tile_near<PARITY, MULTIPHASE, S>(phys, m, t, ring);
+    else batch_tile<PARITY, false, MULTIPHASE, S>(phys, m, t, ring);
 }
 
 // One word per 32 x 4 column and 32 planes: bit k set if a cell of the column in plane 32 g + k is solid or has
@@ -1588,7 +1601,7 @@ dim3 cs_grid(const KParams& kp) {
 // Launch of a step kernel, whose blocks may start before the previous kernel of the stream has finished and
 // wait for it in dep_wait().
 template <class... KA, class... A>
-cudaError_t launch_dep(void (*kernel)(KA...), dim3 g, dim3 b, cudaStream_t st, A... args) {
+cudaError_t launch_dep(void (*kernel)(KA...), dim3 g, dim3 b, cudaStream_t st, const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = g;
     cfg.blockDim = b;
@@ -1598,7 +1611,7 @@ cudaError_t launch_dep(void (*kernel)(KA...), dim3 g, dim3 b, cudaStream_t st, A
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KA(args)...);
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
 }
 
 // Launches one collide_kernel instantiation (internal linkage: each lattice's translation unit
@@ -1675,33 +1688,21 @@ void launch_gather_store(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, int
     else gather_kernel<1, true, F16><<<g, b, 0, st>>>(kp, B.f, B.nbmask, out, B.rsrc);
 }
 
-// multi-domain launch helpers (internal linkage: each lattice's translation unit launches its own kernels)
+// multi-domain launch helper (internal linkage: each lattice's translation unit launches its own kernels)
 template <int S>
 cudaError_t launch_collide_batch_shape(const KParams& phys, const BatchDomTable& doms, const BatchTile* tiles,
                                        int ntiles, int key, cudaStream_t st) {
-    const dim3 b(BATCH_SHAPES[S].bx, BATCH_SHAPES[S].by);
+    const dim3 g(ntiles), b(BATCH_SHAPES[S].bx, BATCH_SHAPES[S].by);
     switch (key) {
-        case 0: collide_batch_kernel<0, false, false, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
-        case 1: collide_batch_kernel<0, false, true, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
-        case 2: collide_batch_kernel<0, true, false, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
-        case 3: collide_batch_kernel<0, true, true, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
-        case 4: collide_batch_kernel<1, false, false, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
-        case 5: collide_batch_kernel<1, false, true, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
-        case 6: collide_batch_kernel<1, true, false, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
-        default: collide_batch_kernel<1, true, true, S><<<ntiles, b, 0, st>>>(phys, doms, tiles); break;
+        case 0: return launch_dep(collide_batch_kernel<0, false, false, S>, g, b, st, phys, doms, tiles);
+        case 1: return launch_dep(collide_batch_kernel<0, false, true, S>, g, b, st, phys, doms, tiles);
+        case 2: return launch_dep(collide_batch_kernel<0, true, false, S>, g, b, st, phys, doms, tiles);
+        case 3: return launch_dep(collide_batch_kernel<0, true, true, S>, g, b, st, phys, doms, tiles);
+        case 4: return launch_dep(collide_batch_kernel<1, false, false, S>, g, b, st, phys, doms, tiles);
+        case 5: return launch_dep(collide_batch_kernel<1, false, true, S>, g, b, st, phys, doms, tiles);
+        case 6: return launch_dep(collide_batch_kernel<1, true, false, S>, g, b, st, phys, doms, tiles);
+        default: return launch_dep(collide_batch_kernel<1, true, true, S>, g, b, st, phys, doms, tiles);
     }
-    return cudaGetLastError();
-}
-
-template <int S>
-cudaError_t launch_psi_batch_shape(const KParams& phys, const BatchDomTable& doms, const BatchTile* tiles, int ntiles,
-                                   int parity, int solids, cudaStream_t st) {
-    const dim3 b(BATCH_SHAPES[S].bx, BATCH_SHAPES[S].by);
-    if (parity == 0 && !solids) psi_batch_kernel<0, false, S><<<ntiles, b, 0, st>>>(phys, doms, tiles);
-    else if (parity == 0) psi_batch_kernel<0, true, S><<<ntiles, b, 0, st>>>(phys, doms, tiles);
-    else if (!solids) psi_batch_kernel<1, false, S><<<ntiles, b, 0, st>>>(phys, doms, tiles);
-    else psi_batch_kernel<1, true, S><<<ntiles, b, 0, st>>>(phys, doms, tiles);
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -1803,10 +1804,10 @@ cudaError_t LBM_CAT(launch_collide_q, LBM_Q)(const KParams& kp, int parity, int 
 }
 
 cudaError_t LBM_CAT(launch_collide_batch_q, LBM_Q)(const KParams& phys, const BatchDomTable& doms,
-                                                   const BatchTile* tiles, int ntiles, int parity, int solids,
+                                                   const BatchTile* tiles, int ntiles, int parity, int near,
                                                    int shape, cudaStream_t st) {
     if (ntiles <= 0) return cudaSuccess;
-    const int key = parity * 4 + (solids ? 2 : 0) + (phys.multiphase ? 1 : 0);
+    const int key = parity * 4 + (near ? 2 : 0) + (phys.multiphase ? 1 : 0);
     switch (shape) {
         case 0: return launch_collide_batch_shape<0>(phys, doms, tiles, ntiles, key, st);
         case 1: return launch_collide_batch_shape<1>(phys, doms, tiles, ntiles, key, st);
@@ -1818,25 +1819,14 @@ cudaError_t LBM_CAT(launch_collide_batch_q, LBM_Q)(const KParams& phys, const Ba
 }
 
 cudaError_t LBM_CAT(launch_psi_runs_q, LBM_Q)(const KParams& phys, const BatchDomTable& doms, const BatchRun* runs,
-                                              int nruns, int parity, cudaStream_t st) {
+                                              int nruns, int parity, int near, cudaStream_t st) {
     if (nruns <= 0) return cudaSuccess;
-    if (parity == 0) psi_run_kernel<0><<<nruns, RUN_NT, 0, st>>>(phys, doms, runs);
-    else psi_run_kernel<1><<<nruns, RUN_NT, 0, st>>>(phys, doms, runs);
-    return cudaGetLastError();
-}
-
-cudaError_t LBM_CAT(launch_psi_batch_q, LBM_Q)(const KParams& phys, const BatchDomTable& doms,
-                                               const BatchTile* tiles, int ntiles, int parity, int solids, int shape,
-                                               cudaStream_t st) {
-    if (ntiles <= 0) return cudaSuccess;
-    switch (shape) {
-        case 0: return launch_psi_batch_shape<0>(phys, doms, tiles, ntiles, parity, solids, st);
-        case 1: return launch_psi_batch_shape<1>(phys, doms, tiles, ntiles, parity, solids, st);
-        case 2: return launch_psi_batch_shape<2>(phys, doms, tiles, ntiles, parity, solids, st);
-        case 3: return launch_psi_batch_shape<3>(phys, doms, tiles, ntiles, parity, solids, st);
-        case 4: return launch_psi_batch_shape<4>(phys, doms, tiles, ntiles, parity, solids, st);
-        default: return cudaErrorInvalidValue;
-    }
+    const dim3 g(nruns), b(RUN_NT);
+    if (parity == 0)
+        return near ? launch_dep(psi_run_kernel<0, true>, g, b, st, phys, doms, runs)
+                    : launch_dep(psi_run_kernel<0, false>, g, b, st, phys, doms, runs);
+    return near ? launch_dep(psi_run_kernel<1, true>, g, b, st, phys, doms, runs)
+                : launch_dep(psi_run_kernel<1, false>, g, b, st, phys, doms, runs);
 }
 
 cudaError_t LBM_CAT(launch_contact_q, LBM_Q)(const KParams& kp, int parity, const Bufs& B, float thr, int* out,

@@ -74,12 +74,13 @@ inline void div_magic(uint32_t d, uint32_t& m, int& s) {
     s = 31 + l;
 }
 
-// A run of cells [begin, end) of member d of a multi-domain launch (cell index (z ny + y) nx + x),
-// none of which needs solid handling: the density/psi pass covers whole planes of a member this way,
-// one block per run, with no lanes left idle at the ends of rows.
+// A run of cells [begin, end) of member d of a multi-domain launch (cell index (z ny + y) nx + x): the
+// density/psi pass covers whole planes of a member this way, one block per run, with no lanes left idle at
+// the ends of rows.  near: some of its planes have cells with solid neighbours.
 struct BatchRun {
     int d;
     uint32_t begin, end;
+    int near;
 };
 
 // Members of one multi-domain launch.  The table travels in the kernel parameters (constant bank),
@@ -93,9 +94,10 @@ struct BatchDomTable {
 // [y0, y0+tile height) x [z0, z0+zc) (clipped to the domain).  narrow = 1: the tile is
 // BATCH_NARROW_BX cells wide and (threads / BATCH_NARROW_BX) high instead of the launch's shape --
 // the last columns of rows whose length leaves at most that many cells past the last full tile.
+// near = 1: some of its cells have solid neighbours.
 constexpr int BATCH_NARROW_BX = 16;
 struct BatchTile {
-    int d, x0, y0, z0, zc, narrow;
+    int d, x0, y0, z0, zc, narrow, near;
 };
 
 // Tile shapes of the multi-domain kernels, compiled for each lattice; lbm_batch_tune picks one per
@@ -143,13 +145,10 @@ struct Bufs {
     cudaError_t launch_gather_q##Q(const KParams& kp, int parity, int solids, const Bufs& B,        \
                                    float* out, cudaStream_t st);                                     \
     cudaError_t launch_collide_batch_q##Q(const KParams& phys, const BatchDomTable& tab,             \
-                                          const BatchTile* tiles, int ntiles, int parity, int solids,  \
+                                          const BatchTile* tiles, int ntiles, int parity, int near,    \
                                           int shape, cudaStream_t st);                                \
-    cudaError_t launch_psi_batch_q##Q(const KParams& phys, const BatchDomTable& tab,                 \
-                                      const BatchTile* tiles, int ntiles, int parity, int solids,      \
-                                      int shape, cudaStream_t st);                                    \
     cudaError_t launch_psi_runs_q##Q(const KParams& phys, const BatchDomTable& tab, const BatchRun* runs, \
-                                     int nruns, int parity, cudaStream_t st);                          \
+                                     int nruns, int parity, int near, cudaStream_t st);                \
     cudaError_t launch_contact_q##Q(const KParams& kp, int parity, const Bufs& B, float thr, int* out, \
                                     cudaStream_t st);                                               \
     cudaError_t launch_onepass_q##Q(const KParams& kp, unsigned* status, cudaStream_t st);          \

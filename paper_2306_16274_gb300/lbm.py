@@ -398,8 +398,8 @@ class Simulation:
 
 
 class Batch:
-    """Many Simulations advanced together (lbm_batch_*): one launch per kernel and group per step,
-    runs of steps replayed from one CUDA graph.  The Simulations stay owned by the caller and must
+    """Many Simulations advanced together (lbm_batch_*): one launch per kernel, lattice and physics per
+    step, runs of steps replayed from CUDA graphs.  The Simulations stay owned by the caller and must
     outlive the Batch."""
 
     def __init__(self, sims, stream=None):
