@@ -168,7 +168,7 @@ inline long long solid_plane_words(const KParams& kp) {
 
 // Lattice-independent kernels (capi.cu)
 cudaError_t launch_nbmask(const KParams& kp, int Q, const uint8_t* solid, uint32_t* nbmask, cudaStream_t st);
-cudaError_t launch_finish_sums(const double* partials, int nblocks, double* sums, cudaStream_t st);
+cudaError_t launch_finish_sums(double* partials, int nblocks, double* sums, cudaStream_t st);
 cudaError_t launch_contact_init(int* out, cudaStream_t st);   // out[6] = 0, 0, INT_MAX, INT_MIN, INT_MAX, INT_MIN
 
 // Sets the message lbm_last_error(NULL) returns on this thread (context-free entry points).
