@@ -727,8 +727,11 @@ __device__ __forceinline__ PairRingSrc pair_ring_src(int w0, int y0, int hx, int
 // density + psi pass over pairs: the counterpart of psi_kernel for the paired layout, one plane per
 // block.  (A z-marching variant with the writers' densities in a shared ring, read at fixed offsets,
 // measured slower: 0.242 against 0.199 ms at 256^3 D3Q19; the per-population reads hit L1.)
+// Without solids for 8 blocks per SM (64 registers): with the compiler's own choice D3Q19 256^3 630.7 against 611.5 us
+// a step, D3Q27 879 against 865; 10 blocks 638 and 975.  With solids the compiler's own choice (0): 400 x 400 x 200
+// 1448 us, 8 blocks 1500, 6 blocks 1482.
 template <int PARITY, bool SOLIDS>
-__global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_pair_kernel(KParams kp, float* __restrict__ psi,
+__global__ void __launch_bounds__(PSI_BX * PSI_BY, SOLIDS ? 0 : 8) psi_pair_kernel(KParams kp, float* __restrict__ psi,
                                                                  unsigned* status, const float* __restrict__ rsrc,
                                                                  float* __restrict__ rdst) {
     const int hx = kp.hx, nx = kp.nx, ny = kp.ny, nz = kp.nz;
