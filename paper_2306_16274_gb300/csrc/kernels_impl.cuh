@@ -78,7 +78,8 @@ constexpr int batch_minb() { return LBM_Q == 19 ? BATCH_SHAPES[S].minb19 : BATCH
 // cells (x, y, z) for z in [z0, z1) of one column: pull the populations (AA phase PARITY),
 // rho = sum f, psi from the equation of state.  F16: the slots hold the shifted FP16 store,
 // read with the densities rsrc they were written with; the new densities go to rdst.
-template <int PARITY, bool SOLIDS, bool F16, class GM, class A>
+// WALLED: the domain has walls or solids (elsewhere than here, where SOLIDS is false)
+template <int PARITY, bool SOLIDS, bool F16, bool WALLED, class GM, class A>
 __device__ __forceinline__ void psi_column(const KParams& kp, const GM& g, const A& addr, float* __restrict__ psi,
                                            const uint32_t* __restrict__ nbmask, unsigned* status, int x, int y,
                                            int z0, int z1, const float* __restrict__ rsrc, float* __restrict__ rdst) {
@@ -105,10 +106,14 @@ __device__ __forceinline__ void psi_column(const KParams& kp, const GM& g, const
         }
         float p[Q];
         gather32<Q, PARITY, SOLIDS>(addr, o, bits, p);
-        if (F16) denorm<Q, SOLIDS>(p, bits, RsOff32{rsrc, o});
         float rho = 0.0f;
+        if (F16 && WALLED) {
+            rho = denorm_sum<Q, SOLIDS>(p, bits, RsOff32{rsrc, o});
+        } else {
+            if (F16) denorm<Q, SOLIDS>(p, bits, RsOff32{rsrc, o});
 #pragma unroll
-        for (int i = 0; i < Q; ++i) rho += p[i];
+            for (int i = 0; i < Q; ++i) rho += p[i];
+        }
         if (F16) rdst[o.c] = rho;
         if (kp.multiphase) psi[bounded(o.c, (unsigned long long)nxy * nz)] = eval_psi(kp, rho, status);
     }
@@ -149,13 +154,11 @@ __global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_kernel(KParams kp, float*
     dep_wait();
     const int x0 = blockIdx.x * PSI_BX, y0 = blockIdx.y * PSI_BY;
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-    // (the FP16 store's densities are summed by one code throughout a domain with solids: the compiler fuses
-    // the products of the two forms differently)
-    if (MIXED && (F16 || SolidPlanes(g, zmask, x0, y0, PSI_BX, PSI_BY, blockIdx.y * gridDim.x + blockIdx.x,
-                                     gridDim.x * gridDim.y).at(z)))
-        psi_column<PARITY, true, F16>(kp, g, addr, psi, nbmask, status, x, y, z, z + 1, rsrc, rdst);
+    if (MIXED && SolidPlanes(g, zmask, x0, y0, PSI_BX, PSI_BY, blockIdx.y * gridDim.x + blockIdx.x,
+                             gridDim.x * gridDim.y).at(z))
+        psi_column<PARITY, true, F16, true>(kp, g, addr, psi, nbmask, status, x, y, z, z + 1, rsrc, rdst);
     else
-        psi_column<PARITY, false, F16>(kp, g, addr, psi, nbmask, status, x, y, z, z + 1, rsrc, rdst);
+        psi_column<PARITY, false, F16, MIXED>(kp, g, addr, psi, nbmask, status, x, y, z, z + 1, rsrc, rdst);
 }
 
 
@@ -727,16 +730,11 @@ __device__ __forceinline__ PairRingSrc pair_ring_src(int w0, int y0, int hx, int
 // density + psi pass over pairs: the counterpart of psi_kernel for the paired layout, one plane per
 // block.  (A z-marching variant with the writers' densities in a shared ring, read at fixed offsets,
 // measured slower: 0.242 against 0.199 ms at 256^3 D3Q19; the per-population reads hit L1.)
-// Without solids for 8 blocks per SM (64 registers): with the compiler's own choice D3Q19 256^3 630.7 against 611.5 us
-// a step, D3Q27 879 against 865; 10 blocks 638 and 975.  With solids the compiler's own choice (0): 400 x 400 x 200
-// 1448 us, 8 blocks 1500, 6 blocks 1482.
-template <int PARITY, bool SOLIDS>
-__global__ void __launch_bounds__(PSI_BX * PSI_BY, SOLIDS ? 0 : 8) psi_pair_kernel(KParams kp, float* __restrict__ psi,
-                                                                 unsigned* status, const float* __restrict__ rsrc,
-                                                                 float* __restrict__ rdst) {
+template <int PARITY, bool SOLIDS, bool WALLED>
+__device__ __forceinline__ void psi_pairs(const KParams& kp, float* __restrict__ psi, unsigned* status,
+                                          const float* __restrict__ rsrc, float* __restrict__ rdst, int z) {
     const int hx = kp.hx, nx = kp.nx, ny = kp.ny, nz = kp.nz;
-    const int w = blockIdx.x * PSI_BX + threadIdx.x, y = blockIdx.y * PSI_BY + threadIdx.y, z = swept_block(kp.down);
-    dep_wait();
+    const int w = blockIdx.x * PSI_BX + threadIdx.x, y = blockIdx.y * PSI_BY + threadIdx.y;
     if (w >= hx || y >= ny) return;
     const uint32_t nxy = (uint32_t)nx * (uint32_t)ny;
     WOff o;
@@ -764,13 +762,34 @@ __global__ void __launch_bounds__(PSI_BX * PSI_BY, SOLIDS ? 0 : 8) psi_pair_kern
         float p[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) p[i] = h ? half_hi(wv[i]) : half_lo(wv[i]);
-        denorm<Q, SOLIDS>(p, bits, RsOff32{rsrc, on[h]});
         float rho = 0.0f;
+        if (WALLED) {
+            rho = denorm_sum<Q, SOLIDS>(p, bits, RsOff32{rsrc, on[h]});
+        } else {
+            denorm<Q, false>(p, 0u, RsOff32{rsrc, on[h]});
 #pragma unroll
-        for (int i = 0; i < Q; ++i) rho += p[i];
+            for (int i = 0; i < Q; ++i) rho += p[i];
+        }
         rdst[on[h].c] = rho;
         if (kp.multiphase) psi[bounded(on[h].c, (unsigned long long)nxy * nz)] = eval_psi(kp, rho, status);
     }
+}
+
+// For 8 blocks per SM (64 registers): with the compiler's own choice D3Q19 256^3 630.7 against 611.5 us a step, D3Q27
+// 879 against 865; 10 blocks 638 and 975.
+// MIXED: solid handling in the planes that SolidPlanes names (no mask in this layout: at walls in y and z).  With it
+// in all planes of a domain with walls / in those alone, us a step: D3Q19 400 x 400 x 200 1448 / 1328, D3Q27
+// 200 x 200 x 100 319 / 289; one slot per cell (psi_kernel) 201 x 200 x 100 219 / 199.
+template <int PARITY, bool MIXED>
+__global__ void __launch_bounds__(PSI_BX * PSI_BY, 8) psi_pair_kernel(const KParams kp, float* __restrict__ psi,
+                                                                    unsigned* status, const float* __restrict__ rsrc,
+                                                                    float* __restrict__ rdst) {
+    const int z = swept_block(kp.down);
+    dep_wait();
+    if (MIXED && SolidPlanes(KGeom{kp}, nullptr, 0, blockIdx.y * PSI_BY, 0, PSI_BY, 0, 0).at(z))
+        psi_pairs<PARITY, true, true>(kp, psi, status, rsrc, rdst, z);
+    else
+        psi_pairs<PARITY, false, MIXED>(kp, psi, status, rsrc, rdst, z);
 }
 
 // Planes [z0, zend) of one tile of pairs; ring: psi (low cells, high cells), rring: the densities the

@@ -252,6 +252,22 @@ __device__ __forceinline__ void denorm(float (&p)[Q], uint32_t bits, const RS& r
     }
 }
 
+// Density of a cell of a domain with walls or solids from its slot values, every rounding written out: cells
+// with and without solid neighbours take different code, and the density must not depend on which.  (Each
+// product is rounded before it is added, but the last.)
+template <int Q, bool SOLIDS, class RS>
+__device__ __forceinline__ float denorm_sum(const float (&p)[Q], uint32_t bits, const RS& rs) {
+    const float self = rs.at(0, 0, 0);
+    float rho = 0.0f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const bool own = i == 0 || (SOLIDS && ((bits >> OPP(i)) & 1u));
+        const float a = __fadd_rn(OMEGA<Q>(i), p[i]), r = own ? self : rs.at(-EX(i), -EY(i), -EZ(i));
+        rho = i < Q - 1 ? __fadd_rn(rho, __fmul_rn(a, r)) : __fmaf_rn(a, r, rho);
+    }
+    return rho;
+}
+
 // ... and populations -> slot values of a cell of density rho
 template <int Q>
 __device__ __forceinline__ void normalize(float (&p)[Q], float rho) {
