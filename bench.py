@@ -328,7 +328,8 @@ def run_batched(steps, n_jobs=64):
         batch_ms = e0.elapsed_time(e1)
         batch.sync()
         info = batch.info()
-        shapes = [g["shape"] for g in batch.groups()]
+        groups = batch.groups()   # groups with and without solid handling share their launches
+        shapes = [g["shape"] for g in groups]
         batch.close()
         for s in sims:
             s.close()
@@ -339,7 +340,7 @@ def run_batched(steps, n_jobs=64):
             "batched": {"mlups": cells * steps / (batch_ms * 1e-3) / 1e6, "ms": batch_ms,
                         "hbm_frac": byts * steps / (batch_ms * 1e-3) / 1e9 / measured_peaks()[0],
                         "groups": info["groups"], "tiles": info["tiles"], "graph_mode": info["graph_mode"],
-                        "zchunk": choice, "tile_shapes": shapes, "launches_per_step": 2 * info["groups"]},
+                        "zchunk": choice, "tile_shapes": shapes, "launches_per_step": 2 * sum(1 for g in groups if not g["solids"])},
             "speedup": loop_ms / batch_ms}
 
 
