@@ -57,6 +57,7 @@ struct Launch {
 struct Chain {
     int Q = 19, plain = -1, solid = -1;   // its groups (solid: -1 if no member has walls or solids)
     std::vector<int> members;
+    std::vector<unsigned long long> masks;   // the members' mask_id when the launches were built
     std::vector<Launch> launches;
 };
 
@@ -265,6 +266,8 @@ int auto_zchunk(const lbm_batch* b, const Chain& c, int resident, int tw, int th
 
 lbm_status build_chain(lbm_batch* b, Chain& c) {
     free_chain(c);
+    c.masks.clear();
+    for (int i : c.members) c.masks.push_back(b->members[i]->mask_id);
     Group& plain = b->groups[c.plain];
     Group* solid = c.solid >= 0 ? &b->groups[c.solid] : nullptr;
     if (plain.shape < 0 || plain.shape >= lbm::BATCH_NSHAPES) return bfail(b, LBM_ERR_ARG, "unknown tile shape");
@@ -442,7 +445,7 @@ lbm_status regroup(lbm_batch* b) {
     return build_chains(b);
 }
 
-// Has any member changed (re-initialised with another solid mask) since the groups were built?
+// Has any member changed (got or lost a solid mask) since the groups were built?
 bool members_changed(const lbm_batch* b) {
     for (size_t i = 0; i < b->members.size(); ++i) {
         const BatchDom d = dom_of(b->members[i]);
@@ -451,6 +454,22 @@ bool members_changed(const lbm_batch* b) {
             return true;
     }
     return false;
+}
+
+// Brings groups, chains and tiles in line with members that were re-initialised: regroups if one got or lost a
+// solid mask, re-tiles the chains with a member whose mask was given anew (it lies in the same buffers, and
+// which planes of a column need solid handling depends on its cells); tuned shapes and z-chunks stay then.
+lbm_status refresh(lbm_batch* b) {
+    if (members_changed(b)) return regroup(b);
+    for (Chain& c : b->chains) {
+        bool same = true;
+        for (size_t j = 0; j < c.members.size(); ++j) same &= c.masks[j] == b->members[c.members[j]]->mask_id;
+        if (!same) {
+            lbm_status s = build_chains(b, c.plain);
+            if (s != LBM_OK) return s;
+        }
+    }
+    return LBM_OK;
 }
 
 // `steps` steps of every member from AA phase `parity` (psi of the current state valid).  Within a chain a step
@@ -557,10 +576,8 @@ lbm_status lbm_batch_step(lbm_batch* b, int32_t n) {
         if (c->parity != parity) return bfail(b, LBM_ERR_STATE, "members were stepped apart: AA phases differ");
         if (c->sticky != LBM_OK) return bfail(b, c->sticky, "a member has a sticky error: " + c->err);
     }
-    if (members_changed(b)) {   // e.g. a member was re-initialised with a solid mask: regroup
-        lbm_status s = regroup(b);
-        if (s != LBM_OK) return s;
-    }
+    lbm_status rs = refresh(b);
+    if (rs != LBM_OK) return rs;
     if (n >= 2 && b->graph_parity != parity) {
         drop_graph(b);
         b->graph_parity = parity;

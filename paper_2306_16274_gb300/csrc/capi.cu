@@ -456,6 +456,7 @@ lbm_status lbm_init_fields(lbm_ctx* c, const float* rho, const float* u, const u
             CK(c, cudaMalloc((void**)&c->solid_dev, std::max<size_t>(n, words)));
             c->bytes += n;
         }
+        ++c->mask_id;
         CK(c, cudaMemcpyAsync(c->solid_dev, solid, n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                               c->stream));
         CK(c, lbm::launch_nbmask(c->kp, c->Q, c->solid_dev, c->nbmask, c->stream));

@@ -31,6 +31,7 @@ struct lbm_ctx {
     float* psi = nullptr;        // ncell floats
     uint32_t* nbmask = nullptr;  // ncell words, only when a solid mask was given
     uint32_t* zmask = nullptr;   // with nbmask: solid_plane_words(kp) words (in solid_dev)
+    unsigned long long mask_id = 0;   // counts the solid masks given; another one may sit in the same buffers
     unsigned* status = nullptr;  // device status word
     double* partials = nullptr;  // moments partial sums (4 per block)
     double* sums = nullptr;      // 4 doubles
