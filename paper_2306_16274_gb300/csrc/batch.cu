@@ -59,6 +59,7 @@ struct Chain {
     std::vector<int> members;
     std::vector<unsigned long long> masks;   // the members' mask_id when the launches were built
     std::vector<Launch> launches;
+    bool built = false;                   // the launches are whole: none may run before (a build may fail half-way)
 };
 
 // Steps of the two graphs a batch replays (the longer one only in calls that replay it four times): a graph
@@ -148,6 +149,7 @@ void free_chain(Chain& c) {
         if (L.runs) cudaFree(L.runs);
     }
     c.launches.clear();
+    c.built = false;
 }
 
 constexpr int ZC_WHOLE = 1 << 30;   // a z-chunk candidate: every column marches through all its planes
@@ -360,6 +362,7 @@ lbm_status build_chain(lbm_batch* b, Chain& c) {
         }
         BCK(b, cudaStreamSynchronize(b->stream));   // t and runs go
     }
+    c.built = true;
     return LBM_OK;
 }
 
@@ -458,12 +461,13 @@ bool members_changed(const lbm_batch* b) {
 
 // Brings groups, chains and tiles in line with members that were re-initialised: regroups if one got or lost a
 // solid mask, re-tiles the chains with a member whose mask was given anew (it lies in the same buffers, and
-// which planes of a column need solid handling depends on its cells); tuned shapes and z-chunks stay then.
+// which planes of a column need solid handling depends on its cells) or that an earlier call failed to build;
+// tuned shapes and z-chunks stay then.
 lbm_status refresh(lbm_batch* b) {
     if (members_changed(b)) return regroup(b);
     for (Chain& c : b->chains) {
-        bool same = true;
-        for (size_t j = 0; j < c.members.size(); ++j) same &= c.masks[j] == b->members[c.members[j]]->mask_id;
+        bool same = c.built;
+        for (size_t j = 0; same && j < c.members.size(); ++j) same = c.masks[j] == b->members[c.members[j]]->mask_id;
         if (!same) {
             lbm_status s = build_chains(b, c.plain);
             if (s != LBM_OK) return s;
