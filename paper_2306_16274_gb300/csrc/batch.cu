@@ -690,6 +690,8 @@ extern "C" {
 lbm_status lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* zchunk_out, int32_t max_groups) {
     if (!b) return LBM_ERR_ARG;
     if (trial_steps < 1) return bfail(b, LBM_ERR_ARG, "trial_steps must be >= 1");
+    lbm_status rs = refresh(b);
+    if (rs != LBM_OK) return rs;
     const int G = (int)b->groups.size();
     std::vector<std::vector<double>> t;
     // stage 1: every tile shape (on all groups at once) with automatic z-chunks; a group and its
@@ -748,6 +750,11 @@ lbm_status lbm_batch_set_group(lbm_batch* b, int32_t group, int32_t shape, int32
     if (group < 0 || group >= (int32_t)b->groups.size()) return bfail(b, LBM_ERR_ARG, "no such group");
     if (shape < 0 || shape >= lbm::BATCH_NSHAPES) return bfail(b, LBM_ERR_ARG, "shape must lie in [0, LBM_BATCH_SHAPES)");
     if (zchunk < 0) return bfail(b, LBM_ERR_ARG, "zchunk must be >= 0");
+    if (members_changed(b)) {   // the chain's tiles may need a group that is not there yet
+        lbm_status s = regroup(b);
+        if (s != LBM_OK) return s;
+        if (group >= (int32_t)b->groups.size()) return bfail(b, LBM_ERR_ARG, "no such group");
+    }
     b->groups[group].shape = shape;
     b->groups[group].zchunk = zchunk;
     const int p = partner_group(b, group);

@@ -252,11 +252,33 @@ void failed_rebuild() {
     }
 }
 
+// A member that needs solid handling since it was last stepped (here: a wall, in use: a mask), tuned or given a
+// shape before it is stepped again: its groups follow first.
+void retiled_after_change(bool tune) {
+    Domains d;
+    d.add(19, 33, 9, 14, false);
+    d.add(27, 33, 9, 14, false);
+    lbm_batch* b = nullptr;
+    REQUIRE(lbm_batch_create(d.ctx.data(), 2, nullptr, &b) == LBM_OK);
+    REQUIRE(lbm_batch_step(b, 2) == LBM_OK);
+    d.ctx[1]->kp.wall_y = 1;
+    if (tune) REQUIRE(lbm_batch_tune(b, 1, nullptr, 0) == LBM_OK);
+    else REQUIRE(lbm_batch_set_group(b, 1, 1, 4) == LBM_OK);
+    int32_t groups = 0;
+    REQUIRE(lbm_batch_info(b, &groups, nullptr, nullptr) == LBM_OK && groups == 3);
+    d.stepped(tune ? 26 : 2);
+    REQUIRE(lbm_batch_step(b, 3) == LBM_OK);
+    d.stepped(tune ? 29 : 5);
+    lbm_batch_destroy(b);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
     const std::string which = argc > 1 ? argv[1] : "";
     if (which == "failed_rebuild") failed_rebuild();
+    else if (which == "tune_after_change") retiled_after_change(true);
+    else if (which == "set_group_after_change") retiled_after_change(false);
     else return 2;
     std::printf("ok\n");
     return 0;
