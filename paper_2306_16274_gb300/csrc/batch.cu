@@ -111,8 +111,7 @@ struct lbm_batch {
     std::vector<Chain> chains;
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;     // capture stream
-    cudaGraphExec_t exec[2] = {nullptr, nullptr};   // GRAPH_STEPS[k] steps from AA phase graph_parity
-    int graph_parity = -1;          // AA phase the graphs were recorded for (-1: none)
+    cudaGraphExec_t exec[2][2] = {};   // [AA phase a call starts from][k]: GRAPH_STEPS[k] steps (nullptr: not recorded)
     std::vector<cudaStream_t> side; // one per chain: the chains run concurrently
     cudaEvent_t fork = nullptr;
     std::vector<cudaEvent_t> done;
@@ -136,11 +135,11 @@ lbm_status bfail(lbm_batch* b, lbm_status s, const std::string& m) {
     } while (0)
 
 void drop_graph(lbm_batch* b) {
-    for (cudaGraphExec_t& e : b->exec) {
-        if (e) cudaGraphExecDestroy(e);
-        e = nullptr;
-    }
-    b->graph_parity = -1;
+    for (auto& phase : b->exec)
+        for (cudaGraphExec_t& e : phase) {
+            if (e) cudaGraphExecDestroy(e);
+            e = nullptr;
+        }
 }
 
 void free_chain(Chain& c) {
@@ -513,7 +512,9 @@ cudaError_t step_all(lbm_batch* b, int parity, int steps, cudaStream_t st) {
     return e;
 }
 
-// b->exec[k]: GRAPH_STEPS[k] steps as one graph
+// b->exec[parity][k]: GRAPH_STEPS[k] steps as one graph.  One set per AA phase: calls of an odd number of steps start
+// from the other phase each time.  Recorded anew whenever the phase changed / kept, us a call of 65 steps: 4 chains of
+// one 24^3 member each 1386 / 903, 24 chains 5230 / 2484; of 5 steps 185 / 93 and 792 / 290.
 lbm_status record_graph(lbm_batch* b, int k, int parity) {
     if (!b->cap) BCK(b, cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
     BCK(b, cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
@@ -521,10 +522,10 @@ lbm_status record_graph(lbm_batch* b, int k, int parity) {
     cudaGraph_t g = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
     if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec[k], g, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec[parity][k], g, 0);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-        b->exec[k] = nullptr;
+        b->exec[parity][k] = nullptr;
         return bfail(b, LBM_ERR_CUDA, std::string("graph: ") + cudaGetErrorString(e));
     }
     return LBM_OK;
@@ -582,18 +583,15 @@ lbm_status lbm_batch_step(lbm_batch* b, int32_t n) {
     }
     lbm_status rs = refresh(b);
     if (rs != LBM_OK) return rs;
-    if (n >= 2 && b->graph_parity != parity) {
-        drop_graph(b);
-        b->graph_parity = parity;
-    }
+    cudaGraphExec_t* exec = b->exec[parity];
     int left = n;
     for (int k = 1; k >= 0; --k) {
-        if (left < GRAPH_STEPS[k] || (k == 1 && !b->exec[1] && n < 4 * GRAPH_STEPS[1])) continue;
-        if (!b->exec[k]) {
+        if (left < GRAPH_STEPS[k] || (k == 1 && !exec[1] && n < 4 * GRAPH_STEPS[1])) continue;
+        if (!exec[k]) {
             lbm_status s = record_graph(b, k, parity);
             if (s != LBM_OK) return s;
         }
-        for (; left >= GRAPH_STEPS[k]; left -= GRAPH_STEPS[k]) BCK(b, cudaGraphLaunch(b->exec[k], b->stream));
+        for (; left >= GRAPH_STEPS[k]; left -= GRAPH_STEPS[k]) BCK(b, cudaGraphLaunch(exec[k], b->stream));
     }
     if (left > 0) BCK(b, step_all(b, parity ^ ((n - left) & 1), left, b->stream));
     advance_members(b, n);
@@ -770,7 +768,7 @@ lbm_status lbm_batch_info(const lbm_batch* b, int32_t* ngroups, int32_t* ntiles,
         for (const Group& g : b->groups) t += g.ntiles;
         *ntiles = (int32_t)std::min<long long>(t, 0x7fffffff);
     }
-    if (graph_mode) *graph_mode = b->graph_parity >= 0 ? 2 : 0;
+    if (graph_mode) *graph_mode = b->exec[0][0] || b->exec[0][1] || b->exec[1][0] || b->exec[1][1] ? 2 : 0;
     return LBM_OK;
 }
 

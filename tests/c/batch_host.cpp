@@ -272,6 +272,29 @@ void retiled_after_change(bool tune) {
     lbm_batch_destroy(b);
 }
 
+// Calls of an odd number of steps begin in the other AA phase each time: graphs are recorded once per phase, not
+// once per call, and every call takes exactly its steps.
+void odd_calls() {
+    for (int n : {2, 3, 5, 7, 19, 33, 65, 67, 129}) {
+        collided.clear();
+        summed.clear();
+        Domains d = three();
+        lbm_batch* b = nullptr;
+        REQUIRE(lbm_batch_create(d.ctx.data(), (int)d.ctx.size(), nullptr, &b) == LBM_OK);
+        instantiated = 0;
+        long long steps = 0;
+        for (int k = 0; k < 12; ++k) {
+            REQUIRE(lbm_batch_step(b, n) == LBM_OK);
+            d.stepped(steps += n);
+        }
+        const int most = (n % 2 ? 2 : 1) * (n >= 64 ? 2 : 1);
+        if (instantiated > most) std::printf("%d graphs for calls of %d steps\n", instantiated, n);
+        REQUIRE(instantiated <= most);
+        lbm_batch_destroy(b);
+        by_base.clear();
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -279,6 +302,7 @@ int main(int argc, char** argv) {
     if (which == "failed_rebuild") failed_rebuild();
     else if (which == "tune_after_change") retiled_after_change(true);
     else if (which == "set_group_after_change") retiled_after_change(false);
+    else if (which == "odd_calls") odd_calls();
     else return 2;
     std::printf("ok\n");
     return 0;
