@@ -433,12 +433,17 @@ __device__ __forceinline__ void collide_tile(const KParams& kp, const GM& g, con
         set_plane(o, z, nz, nxy);
         if (bits & 1u) continue;
 #else
-        static_assert(SOLIDS != 2, "mixed tiles gather a plane ahead");
         set_plane(o, z, nz, nxy);
-        const uint32_t bits = SOLIDS ? solid_bits32<Q>(g, nbmask, o.c, x, y, z) : 0u;
-        if (bits & 1u) continue;
         float p[Q];
-        gather32<Q, PARITY, SOLIDS>(addr, o, bits, p);
+        uint32_t bits = 0u;
+        [[maybe_unused]] bool near = false;
+        if constexpr (SOLIDS == 2) {
+            near = gather_mixed<PARITY>(g, addr, o, nbmask, sp, x, y, z, bits, p);
+        } else {
+            bits = SOLIDS ? solid_bits32<Q>(g, nbmask, o.c, x, y, z) : 0u;
+            if (!(bits & 1u)) gather32<Q, PARITY, SOLIDS>(addr, o, bits, p);
+        }
+        if (bits & 1u) continue;
 #endif
         float rho, ux, uy, uz;
         if constexpr (SOLIDS == 2) {
