@@ -49,7 +49,8 @@ struct Launch {
     BatchDomTable tab{};
     BatchTile* tiles = nullptr;     // device
     BatchRun* runs = nullptr;       // device
-    int nt = 0, nr = 0, near = 0;   // near: some tile or run has cells with solid neighbours
+    int nt = 0, nr = 0;
+    int near = lbm::NEAR_NONE;      // which tiles and runs have cells with solid neighbours
 };
 
 // A chain: the members of one lattice and physics, advanced by their own sequence of launches.  Their tiles
@@ -191,19 +192,22 @@ lbm_status member_tile_flags(lbm_batch* b, lbm_ctx* c, int tw, int th) {
     return LBM_OK;
 }
 
-// Tiles of the members of a chain: tw x th cells in (x, y) (the groups' shape) and a run of z planes.  Along every
-// column the planes are split into runs that need solid handling (a cell with a solid neighbour:
-// mask, or the first / last plane, row or column next to a wall) and runs that do not; runs are
-// cut into chunks of at most zc planes (the group's fixed zchunk, a member's own, or automatic).  Only the
-// tiles with solid neighbours pay for the solid tests.
+// Tiles of the members of a chain: tw x th cells in (x, y) (the groups' shape) and a chunk of at most zc z planes (the
+// group's fixed zchunk, a member's own, or automatic).  A tile with planes that need solid handling (a cell with
+// a solid neighbour: mask, or the first / last plane, row or column next to a wall) names them in its bits, and
+// its march switches from plane to plane; only those planes pay for the solid tests.  (As marches of their own
+// they paid for their start, too: figures at collide_batch_kernel.)  The first and the last plane of a column are tiles of
+// their own where the plane beside them needs no solid handling, as at walls in z: four 40^3 domains 16.4 us a step
+// (D3Q19) and 22.4 (D3Q27) so, 17.6 and 28.4 as part of the column's first and last chunks.
 //
 // Where a row leaves 1 .. 16 cells past its last full tile width (tw = 32), those cells form narrow
 // columns, 16 cells wide and twice as high, which the same blocks step (BatchTile::narrow): a
 // 32-wide tile there would leave 16 to 31 of its 32 lanes per row idle.
 //
 // The density/psi pass covers a member as runs of consecutive cells of whole planes: it needs no stencil, so
-// nothing ties its threads to rows, and rows that do not fill a tile's width leave no lanes idle.  Planes in
-// which some column has solid neighbours form runs of their own.
+// nothing ties its threads to rows, and rows that do not fill a tile's width leave no lanes idle.  Rows, th
+// at a time, in which some column has solid neighbours form runs of their own.  us a step of four 96^3 domains
+// with a post along z, runs with and without by planes / by rows: D3Q19 153 / 145, D3Q27 221 / 212.
 #ifndef LBM_BATCH_NARROW
 #define LBM_BATCH_NARROW 1
 #endif
@@ -281,7 +285,7 @@ lbm_status build_chain(lbm_batch* b, Chain& c) {
     // 2048 cells a run, fewer where that would leave SMs without their eight blocks
     const uint32_t run_cells = 256u * (uint32_t)std::min(8.0, std::max(1.0, cells / (152.0 * 8.0 * 256.0)));
     std::vector<uint8_t> need;      // per plane of one column: needs solid handling
-    std::vector<uint8_t> mixed;     // per plane: some column needs solid handling
+    std::vector<uint8_t> rows;      // per plane and th rows: some column needs solid handling
     for (size_t j0 = 0; j0 < c.members.size(); j0 += lbm::BATCH_LAUNCH_DOMS) {
         const int nd = (int)std::min(c.members.size() - j0, (size_t)lbm::BATCH_LAUNCH_DOMS);
         c.launches.emplace_back();
@@ -302,7 +306,8 @@ lbm_status build_chain(lbm_batch* b, Chain& c) {
             const int zc[2] = {chunk(plain), chunk(solid ? *solid : plain)};
             const int nxf = (k.nx + fw - 1) / fw, nyf = (k.ny + fh - 1) / fh;
             need.resize(k.nz);
-            mixed.assign(k.nz, 0);
+            const int nrow = (k.ny + th - 1) / th;
+            rows.assign((size_t)nrow * k.nz, 0);
             const size_t member_t0 = t.size();
             for (const Column& col : member_columns(k, tw, th)) {
                 const bool side = (k.wall_x && (col.x0 == 0 || col.x0 + col.w >= k.nx)) ||
@@ -316,30 +321,47 @@ lbm_status build_chain(lbm_batch* b, Chain& c) {
                             for (int fx = fx0; fx < fx1 && !s2; ++fx)
                                 s2 = ctx->tile_flags[((size_t)z * nyf + fy) * nxf + fx] != 0;
                     need[z] = s2 ? 1 : 0;
-                    mixed[z] |= need[z];
+                    for (int y = col.y0; s2 && y < std::min(col.y0 + col.h, k.ny); y += th) rows[(size_t)z * nrow + y / th] = 1;
                 }
-                for (int z0 = 0; z0 < k.nz;) {
-                    int z1 = z0 + 1;
-                    while (z1 < k.nz && need[z1] == need[z0] && z1 - z0 < zc[need[z0]]) ++z1;
-                    t.push_back({d, col.x0, col.y0, z0, z1 - z0, col.narrow, need[z0]});
-                    (need[z0] ? *solid : plain).ntiles += 1;
-                    L.near |= need[z0];
-                    z0 = z1;
+                auto tile = [&](int z0, int n, uint32_t near) {
+                    t.push_back({d, col.x0, col.y0, z0, n, col.narrow, near});
+                    (near ? *solid : plain).ntiles += 1;
+                };
+                auto any = [&](int z0, int n) { return std::find(&need[z0], &need[z0] + n, 1) != &need[z0] + n; };
+                const int first = k.nz > 1 && need[0] && !need[1] ? 1 : 0;
+                const int last = k.nz - (k.nz > 2 && need[k.nz - 1] && !need[k.nz - 2] ? 1 : 0);
+                if (first) tile(0, 1, 1u);
+                for (int z0 = first; z0 < last;) {
+                    int n = std::min(zc[0], last - z0);
+                    uint32_t near = 0;
+                    if (any(z0, n)) {   // by the solid group's z-chunk
+                        n = std::min(std::min(zc[1], 32), last - z0);
+                        for (int j = 0; j < n; ++j) near |= (uint32_t)need[z0 + j] << j;
+                    }
+                    tile(z0, n, near);
+                    if (near) L.near = lbm::NEAR_SOME;
+                    z0 += n;
                 }
+                if (last < k.nz) tile(last, 1, 1u);
+                if ((first || last < k.nz) && L.near == lbm::NEAR_NONE) L.near = lbm::NEAR_ENDS;
             }
             // z-chunk-major order within the member (as the single-domain grid): blocks resident at
             // the same time work on neighbouring columns of the same planes
             std::stable_sort(t.begin() + member_t0, t.end(), [](const BatchTile& a, const BatchTile& b2) {
                 return a.z0 != b2.z0 ? a.z0 < b2.z0 : (a.y0 != b2.y0 ? a.y0 < b2.y0 : a.x0 < b2.x0);
             });
-            const uint32_t nxy = (uint32_t)k.nx * (uint32_t)k.ny;
-            for (int z0 = 0; z0 < k.nz;) {
-                int z1 = z0 + 1;
-                while (z1 < k.nz && mixed[z1] == mixed[z0]) ++z1;
-                const uint32_t end = (uint32_t)z1 * nxy;
-                for (uint32_t a = (uint32_t)z0 * nxy; a < end; a += std::min(run_cells, end - a))
-                    runs.push_back({d, a, a + std::min(run_cells, end - a), mixed[z0]});
-                z0 = z1;
+            // the rows in the order of the cells: those before block j of th rows
+            auto cells_before = [&](int j) {
+                return ((uint32_t)(j / nrow) * (uint32_t)k.ny + (uint32_t)(j % nrow * th)) * (uint32_t)k.nx;
+            };
+            const int blocks = nrow * k.nz;
+            for (int j0 = 0; j0 < blocks;) {
+                int j1 = j0 + 1;
+                while (j1 < blocks && rows[j1] == rows[j0]) ++j1;
+                const uint32_t end = cells_before(j1);
+                for (uint32_t a = cells_before(j0); a < end; a += std::min(run_cells, end - a))
+                    runs.push_back({d, a, a + std::min(run_cells, end - a), rows[j0]});
+                j0 = j1;
             }
         }
         // longest marches first within a launch: blocks start roughly in index order, so the short ones
@@ -349,6 +371,11 @@ lbm_status build_chain(lbm_batch* b, Chain& c) {
         // against the collide pass's direction: the pass starts on what that one left in the L2
         std::reverse(runs.begin(), runs.end());
         if (t.size() > 0x7fffffff || runs.size() > 0x7fffffff) return bfail(b, LBM_ERR_ARG, "too many tiles");
+        // Wall planes in a kernel whose plain tiles keep their registers, or in one that takes any tile: the latter
+        // is faster on D3Q27 in launches of many waves (us a step with walls in z: four 96^3, 3744 tiles, 220.9 / 218.8, ten of
+        // 48^3 - 102^3 311.8 / 305.6; but four 72^3, 3060 tiles, 101.6 / 104.0 and four 40^3 21.3 / 22.4; D3Q19 four 96^3
+        // 147.4 / 149.1).
+        if (L.near == lbm::NEAR_ENDS && c.Q == 27 && t.size() > 4.5 * 152.0 * sh.minb27) L.near = lbm::NEAR_SOME;
         L.nt = (int)t.size();
         L.nr = (int)runs.size();
         if (L.nt > 0) {

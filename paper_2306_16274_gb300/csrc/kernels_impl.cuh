@@ -43,6 +43,13 @@ struct SolidPlanes {
     }
 };
 
+// The same of a multi-domain tile: bit k for plane z0 + k.
+struct TilePlanes {
+    uint32_t bits;
+    int z0;
+    __device__ __forceinline__ bool at(int z) const { return (bits >> (z - z0)) & 1u; }
+};
+
 // Marches a chunk [z0, z1) of a column as runs of planes with and without solid neighbours: a run starts
 // its own march (two psi planes and a first plane that nothing overlaps), which only the columns and chunks
 // at solids pay.  The ring is free again for a run once every thread has left the one before it.
@@ -164,7 +171,7 @@ __global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_kernel(KParams kp, float*
 
 // multi-domain density + psi pass over runs of whole planes: thread k of a block takes cells begin + k,
 // begin + k + RUN_NT, ... of its run, so rows of any length pack the warps densely.  Per cell the
-// arithmetic and its order are psi_column's.  A run of planes without solid neighbours takes the code without
+// arithmetic and its order are psi_column's.  A run of rows without solid neighbours takes the code without
 // solid tests.
 constexpr int RUN_NT = 256;
 __device__ __forceinline__ uint32_t div_by_magic(uint32_t n, uint32_t m, int s) {
@@ -289,9 +296,9 @@ __device__ __forceinline__ void put_psi_plane(float* slot, const float (&v)[TS::
 
 // the parts of a mixed tile's cell (SOLIDS == 2 below): its populations and solid bits, returning whether
 // the tile has solid neighbours in plane z ...
-template <int PARITY, class GM, class A>
+template <int PARITY, class GM, class A, class SP>
 __device__ __forceinline__ bool gather_mixed(const GM& g, const A& addr, const Off32& o,
-                                             const uint32_t* __restrict__ nbmask, SolidPlanes& sp, int x, int y, int z,
+                                             const uint32_t* __restrict__ nbmask, SP& sp, int x, int y, int z,
                                              uint32_t& bits, float (&p)[Q]) {
     if (sp.at(z)) {
         bits = solid_bits32<Q>(g, nbmask, o.c, x, y, z);
@@ -327,17 +334,17 @@ __device__ __forceinline__ void cell_forces(const KParams& kp, float (&p)[Q], co
 // with (rsrc) follow the march in a second shared ring `rring`; outputs are written relative
 // to the cell's current density rown.
 // SOLIDS: 0 no cell of the tile has a solid neighbour, 1 every cell is tested, 2 the cells of the planes that
-// sp names (the march switches from plane to plane; only for whole-grid tiles).
+// sp names (the march switches from plane to plane).
 // PSI_PF: the psi (and FP16 density) ring planes are loaded into registers one plane ahead and
-// stored into the ring at the next plane (all but the multi-domain kernels' solid tiles, which
-// have no registers to spare and load each plane just before its barrier).
+// stored into the ring at the next plane (all but the multi-domain kernels' tiles of single wall planes,
+// which have no next plane).
 template <class TS, int PARITY, int SOLIDS, bool MULTIPHASE, bool F16, bool PSI_PF, class GM, class A,
-          bool FLAT = false>
+          bool FLAT = false, class SP = SolidPlanes>
 __device__ __forceinline__ void collide_tile(const KParams& kp, const GM& g, const A& addr, const float* __restrict__ psi,
                                              const uint32_t* __restrict__ nbmask, unsigned* status, int x0, int y0,
                                              int z0, int zchunk, int zmax, float (*ring)[TS::RP], float (*rring)[TS::RP],
                                              const float* __restrict__ rsrc, const float* __restrict__ rown,
-                                             SolidPlanes sp = SolidPlanes()) {
+                                             SP sp = SP()) {
     // FLAT: the block has another shape with as many threads (a narrow multi-domain tile); its threads
     // take the tile's cells in row-major order
     const int tid = FLAT ? (int)(threadIdx.x + blockDim.x * threadIdx.y) : (int)(threadIdx.x + TS::BX * threadIdx.y);
@@ -504,7 +511,6 @@ __device__ __noinline__ void collide_tile_near(const KParams& kp, const float* p
 // as two launches a pass over tile lists, replayed from a graph / as one kernel: D3Q19 127 x 127 x 106 92.5 /
 // 77.8, 256^3 746 / 672, D3Q27 127 x 127 x 106 130.9 / 107.1.  (As a march cut into runs with and without solids,
 // each through its own copy of the tile: 87.9, 709 and 127.6 us; registers spill in the plain copy.)
-enum { NEAR_NONE = 0, NEAR_ENDS = 1, NEAR_SOME = 2 };
 template <int PARITY, int NEAR, bool MULTIPHASE, bool F16>
 __global__ void __launch_bounds__(ZmTile::NT, ZM_MINB) collide_kernel(const __grid_constant__ KParams kp,
                                                                 const float* __restrict__ psi,
@@ -1291,34 +1297,42 @@ __global__ void pull_store_kernel(KParams kp, const float* __restrict__ fin, lon
     }
 }
 
-// one tile of a multi-domain collide-stream pass: of shape S of BATCH_SHAPES, or narrow
-template <int PARITY, bool SOLIDS, bool MULTIPHASE, int S>
+// one tile of a multi-domain collide-stream pass: of shape S of BATCH_SHAPES, or narrow (SOLIDS as in collide_tile)
+template <int PARITY, int SOLIDS, bool MULTIPHASE, int S>
 __device__ __forceinline__ void batch_tile(const KParams& phys, const BatchDom& m, const BatchTile& t,
                                            float (*ring)[BatchTileShape<S>::RP]) {
     using TS = BatchTileShape<S>;
     using TN = TileShape<BATCH_NARROW_BX, TS::NT / BATCH_NARROW_BX>;   // narrow tiles at the ends of rows
     static_assert(TN::RP <= TS::RP, "a narrow tile's ring fits the block's");
+    constexpr bool PSI_PF = SOLIDS != 1;
     const DGeom g{m};
     const DomPlanes addr{m};
+    const TilePlanes sp{t.near, t.z0};
     if (TS::BX != BATCH_NARROW_BX && t.narrow)
-        collide_tile<TN, PARITY, SOLIDS, MULTIPHASE, false, !SOLIDS, DGeom, DomPlanes, true>(
+        collide_tile<TN, PARITY, SOLIDS, MULTIPHASE, false, PSI_PF, DGeom, DomPlanes, true, TilePlanes>(
             phys, g, addr, m.psi, m.nbmask, m.status, t.x0, t.y0, t.z0, t.zc, g.nz(),
-            reinterpret_cast<float (*)[TN::RP]>(&ring[0][0]), nullptr, nullptr, nullptr);
+            reinterpret_cast<float (*)[TN::RP]>(&ring[0][0]), nullptr, nullptr, nullptr, sp);
     else
-        collide_tile<TS, PARITY, SOLIDS, MULTIPHASE, false, !SOLIDS>(phys, g, addr, m.psi, m.nbmask, m.status, t.x0,
-                                                                    t.y0, t.z0, t.zc, g.nz(), ring, nullptr, nullptr,
-                                                                    nullptr);
+        collide_tile<TS, PARITY, SOLIDS, MULTIPHASE, false, PSI_PF, DGeom, DomPlanes, false, TilePlanes>(
+            phys, g, addr, m.psi, m.nbmask, m.status, t.x0, t.y0, t.z0, t.zc, g.nz(), ring, nullptr, nullptr, nullptr, sp);
 }
-// tiles with solid neighbours as a function of their own (see collide_tile_near)
+// a wall's plane as a function of its own (see collide_tile_near)
 template <int PARITY, bool MULTIPHASE, int S>
 __device__ __noinline__ void batch_tile_near(const KParams& phys, const BatchDom& m, const BatchTile& t,
                                              float (*ring)[BatchTileShape<S>::RP]) {
-    batch_tile<PARITY, true, MULTIPHASE, S>(phys, m, t, ring);
+    batch_tile<PARITY, 1, MULTIPHASE, S>(phys, m, t, ring);
 }
 
 // multi-domain collide-stream pass: one block per tile of any member of the launch's table; physics by
-// value.  NEAR: some tiles of the launch have cells with solid neighbours (BatchTile::near).
-template <int PARITY, bool NEAR, bool MULTIPHASE, int S>
+// value.  NEAR: which tiles of the launch have planes with solid neighbours (BatchTile::near) -- NEAR_NONE: none;
+// NEAR_ENDS: single planes next to walls in z; NEAR_SOME: any, and such a tile's march switches from plane to plane.
+// The plain tiles' registers bound the kernel; NEAR_ENDS keeps them whole by calling a function that spills
+// (212 bytes on the even phase of D3Q27, 592 on the odd), which only single planes can afford.  us a step of members with walls
+// or solids, every run of near planes as a march of its own through that function / this: cylinders D3Q19 127 x 127 x
+// 106 91.3 / 82.1, D3Q27 143.4 / 118.3, eight on both lattices, 64 - 160 wide, 739 / 636; walls in x, four 96^3 D3Q19 201
+// / 177; in x and y, four 80 x 96 x 70 D3Q27 221 / 203.  (All tiles of such a launch through the switching march:
+// 85.7 and 118.8 for the first two, but 161 against 153 for four 96^3 with a post, and 226 against 221 for walls in z.)
+template <int PARITY, int NEAR, bool MULTIPHASE, int S>
 __global__ void __launch_bounds__(BatchTileShape<S>::NT, batch_minb<S>()) collide_batch_kernel(
         const __grid_constant__ KParams phys, const __grid_constant__ BatchDomTable tab,
         const BatchTile* __restrict__ tiles) {
@@ -1326,8 +1340,12 @@ __global__ void __launch_bounds__(BatchTileShape<S>::NT, batch_minb<S>()) collid
     const BatchTile t = tiles[blockIdx.x];
     const BatchDom& m = tab.d[t.d];
     dep_wait();
-    if (NEAR && t.near) batch_tile_near<PARITY, MULTIPHASE, S>(phys, m, t, ring);
-    else batch_tile<PARITY, false, MULTIPHASE, S>(phys, m, t, ring);
+    if (NEAR != NEAR_NONE && t.near) {
+        if (NEAR == NEAR_SOME) batch_tile<PARITY, 2, MULTIPHASE, S>(phys, m, t, ring);
+        else batch_tile_near<PARITY, MULTIPHASE, S>(phys, m, t, ring);
+    } else {
+        batch_tile<PARITY, 0, MULTIPHASE, S>(phys, m, t, ring);
+    }
 }
 
 // One word per 32 x 4 column and 32 planes: bit k set if a cell of the column in plane 32 g + k is solid or has
@@ -1722,21 +1740,23 @@ void launch_gather_store(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, int
     else gather_kernel<1, true, F16><<<g, b, 0, st>>>(kp, B.f, B.nbmask, out, B.rsrc);
 }
 
-// multi-domain launch helper (internal linkage: each lattice's translation unit launches its own kernels)
+// multi-domain launch helpers (internal linkage: each lattice's translation unit launches its own kernels)
+template <int NEAR, int S>
+cudaError_t launch_collide_batch_near(dim3 g, dim3 b, const KParams& phys, const BatchDomTable& doms,
+                                      const BatchTile* tiles, int parity, cudaStream_t st) {
+    if (parity == 0)
+        return phys.multiphase ? launch_dep(collide_batch_kernel<0, NEAR, true, S>, g, b, st, phys, doms, tiles)
+                               : launch_dep(collide_batch_kernel<0, NEAR, false, S>, g, b, st, phys, doms, tiles);
+    return phys.multiphase ? launch_dep(collide_batch_kernel<1, NEAR, true, S>, g, b, st, phys, doms, tiles)
+                           : launch_dep(collide_batch_kernel<1, NEAR, false, S>, g, b, st, phys, doms, tiles);
+}
 template <int S>
 cudaError_t launch_collide_batch_shape(const KParams& phys, const BatchDomTable& doms, const BatchTile* tiles,
-                                       int ntiles, int key, cudaStream_t st) {
+                                       int ntiles, int parity, int near, cudaStream_t st) {
     const dim3 g(ntiles), b(BATCH_SHAPES[S].bx, BATCH_SHAPES[S].by);
-    switch (key) {
-        case 0: return launch_dep(collide_batch_kernel<0, false, false, S>, g, b, st, phys, doms, tiles);
-        case 1: return launch_dep(collide_batch_kernel<0, false, true, S>, g, b, st, phys, doms, tiles);
-        case 2: return launch_dep(collide_batch_kernel<0, true, false, S>, g, b, st, phys, doms, tiles);
-        case 3: return launch_dep(collide_batch_kernel<0, true, true, S>, g, b, st, phys, doms, tiles);
-        case 4: return launch_dep(collide_batch_kernel<1, false, false, S>, g, b, st, phys, doms, tiles);
-        case 5: return launch_dep(collide_batch_kernel<1, false, true, S>, g, b, st, phys, doms, tiles);
-        case 6: return launch_dep(collide_batch_kernel<1, true, false, S>, g, b, st, phys, doms, tiles);
-        default: return launch_dep(collide_batch_kernel<1, true, true, S>, g, b, st, phys, doms, tiles);
-    }
+    return near == NEAR_NONE   ? launch_collide_batch_near<NEAR_NONE, S>(g, b, phys, doms, tiles, parity, st)
+           : near == NEAR_ENDS ? launch_collide_batch_near<NEAR_ENDS, S>(g, b, phys, doms, tiles, parity, st)
+                               : launch_collide_batch_near<NEAR_SOME, S>(g, b, phys, doms, tiles, parity, st);
 }
 
 }  // namespace
@@ -1841,13 +1861,12 @@ cudaError_t LBM_CAT(launch_collide_batch_q, LBM_Q)(const KParams& phys, const Ba
                                                    const BatchTile* tiles, int ntiles, int parity, int near,
                                                    int shape, cudaStream_t st) {
     if (ntiles <= 0) return cudaSuccess;
-    const int key = parity * 4 + (near ? 2 : 0) + (phys.multiphase ? 1 : 0);
     switch (shape) {
-        case 0: return launch_collide_batch_shape<0>(phys, doms, tiles, ntiles, key, st);
-        case 1: return launch_collide_batch_shape<1>(phys, doms, tiles, ntiles, key, st);
-        case 2: return launch_collide_batch_shape<2>(phys, doms, tiles, ntiles, key, st);
-        case 3: return launch_collide_batch_shape<3>(phys, doms, tiles, ntiles, key, st);
-        case 4: return launch_collide_batch_shape<4>(phys, doms, tiles, ntiles, key, st);
+        case 0: return launch_collide_batch_shape<0>(phys, doms, tiles, ntiles, parity, near, st);
+        case 1: return launch_collide_batch_shape<1>(phys, doms, tiles, ntiles, parity, near, st);
+        case 2: return launch_collide_batch_shape<2>(phys, doms, tiles, ntiles, parity, near, st);
+        case 3: return launch_collide_batch_shape<3>(phys, doms, tiles, ntiles, parity, near, st);
+        case 4: return launch_collide_batch_shape<4>(phys, doms, tiles, ntiles, parity, near, st);
         default: return cudaErrorInvalidValue;
     }
 }

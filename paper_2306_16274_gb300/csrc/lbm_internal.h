@@ -76,7 +76,7 @@ inline void div_magic(uint32_t d, uint32_t& m, int& s) {
 
 // A run of cells [begin, end) of member d of a multi-domain launch (cell index (z ny + y) nx + x): the
 // density/psi pass covers whole planes of a member this way, one block per run, with no lanes left idle at
-// the ends of rows.  near: some of its planes have cells with solid neighbours.
+// the ends of rows.  near: some of its cells have solid neighbours.
 struct BatchRun {
     int d;
     uint32_t begin, end;
@@ -94,10 +94,12 @@ struct BatchDomTable {
 // [y0, y0+tile height) x [z0, z0+zc) (clipped to the domain).  narrow = 1: the tile is
 // BATCH_NARROW_BX cells wide and (threads / BATCH_NARROW_BX) high instead of the launch's shape --
 // the last columns of rows whose length leaves at most that many cells past the last full tile.
-// near = 1: some of its cells have solid neighbours.
+// near: bit k is set if some of its cells in plane z0 + k are solid or have solid neighbours; a tile with such
+// planes is at most 32 planes high.
 constexpr int BATCH_NARROW_BX = 16;
 struct BatchTile {
-    int d, x0, y0, z0, zc, narrow, near;
+    int d, x0, y0, z0, zc, narrow;
+    uint32_t near;
 };
 
 // Tile shapes of the multi-domain kernels, compiled for each lattice; lbm_batch_tune picks one per
@@ -110,6 +112,9 @@ struct BatchShape {
 constexpr int BATCH_NSHAPES = 5;
 constexpr BatchShape BATCH_SHAPES[BATCH_NSHAPES] = {
     {32, 4, 7, 5}, {32, 2, 14, 10}, {16, 8, 7, 5}, {16, 4, 14, 10}, {32, 4, 6, 4}};
+
+// Which cells of a launch have solid neighbours (collide_kernel, collide_batch_kernel).
+enum { NEAR_NONE = 0, NEAR_ENDS = 1, NEAR_SOME = 2 };
 
 // Device buffers of one context's launches.  f: the population slots, floats or (f16) the
 // shifted FP16 store; rsrc: the densities the stored slots were written with; rnew: the other

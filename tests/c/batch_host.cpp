@@ -5,6 +5,7 @@
 // No GPU is touched.  Usage: batch_host <scenario>; prints "ok" and exits 0.
 #include <cuda_runtime_api.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -33,7 +34,7 @@ struct Pass {
     bool collide;
     lbm::BatchDomTable tab;
     const void* items;
-    int n, parity, shape;
+    int n, parity, shape, near;
 };
 struct Graph {
     std::vector<Pass> passes;
@@ -42,6 +43,30 @@ Graph* capture = nullptr;
 
 std::map<const float*, lbm_ctx*> by_base;
 std::map<const float*, long long> collided, summed;   // cells
+
+bool check_near = false;
+
+// next to a wall of its domain (no member has a mask)
+bool at_wall(const lbm::BatchDom& d, int x, int y, int z) {
+    return (d.wall_x && (x == 0 || x == d.nx - 1)) || (d.wall_y && (y == 0 || y == d.ny - 1)) ||
+           (d.wall_z && (z == 0 || z == d.nz - 1));
+}
+void check_tile(const Pass& p, const lbm::BatchTile& t, const lbm::BatchDom& d, int w, int h) {
+    const int n = std::min(t.zc, d.nz - t.z0);
+    REQUIRE(t.near == 0 || (p.near != lbm::NEAR_NONE && n <= 32 && (n == 32 || t.near >> n == 0)));
+    REQUIRE(t.near == 0 || p.near == lbm::NEAR_SOME || n == 1);
+    for (int j = 0; j < n; ++j) {
+        bool need = false;
+        for (int y = t.y0; y < std::min(t.y0 + h, d.ny); ++y)
+            for (int x = t.x0; x < std::min(t.x0 + w, d.nx); ++x) need |= at_wall(d, x, y, t.z0 + j);
+        REQUIRE(need == (j < 32 && ((t.near >> j) & 1u)));
+    }
+}
+void check_run(const Pass& p, const lbm::BatchRun& r, const lbm::BatchDom& d) {
+    REQUIRE(!r.near || p.near);
+    for (int c = (int)r.begin; c < (int)r.end && !r.near; ++c)
+        REQUIRE(!at_wall(d, c % d.nx, c / d.nx % d.ny, c / d.nx / d.ny));
+}
 
 void check(const Pass& p) {
     const size_t item = p.collide ? sizeof(lbm::BatchTile) : sizeof(lbm::BatchRun);
@@ -63,6 +88,7 @@ void check(const Pass& p) {
             REQUIRE(p.parity == (int)(collided[d.base] / n % 2));
             REQUIRE(collided[d.base] / n == summed[d.base] / n && summed[d.base] % n == 0);
             collided[d.base] += cells;
+            if (check_near) check_tile(p, t, d, w, h);
         } else {
             const lbm::BatchRun& r = ((const lbm::BatchRun*)p.items)[k];
             const lbm::BatchDom& d = p.tab.d[r.d];
@@ -71,6 +97,7 @@ void check(const Pass& p) {
             REQUIRE(r.end <= n && collided[d.base] % n == 0);
             REQUIRE(p.parity == (int)(collided[d.base] / n % 2));
             summed[d.base] += r.end - r.begin;
+            if (check_near) check_run(p, r, d);
         }
     }
 }
@@ -151,12 +178,12 @@ namespace lbm {
 void set_thread_error(const char*) {}
 #define FAKE_LAUNCHERS(Q)                                                                                      \
     cudaError_t launch_collide_batch_q##Q(const KParams&, const BatchDomTable& tab, const BatchTile* t, int n, \
-                                          int parity, int, int shape, cudaStream_t) {                          \
-        return enqueue({true, tab, t, n, parity, shape});                                                      \
+                                          int parity, int near, int shape, cudaStream_t) {                     \
+        return enqueue({true, tab, t, n, parity, shape, near});                                                \
     }                                                                                                          \
     cudaError_t launch_psi_runs_q##Q(const KParams&, const BatchDomTable& tab, const BatchRun* r, int n,       \
-                                     int parity, int, cudaStream_t) {                                          \
-        return enqueue({false, tab, r, n, parity, 0});                                                         \
+                                     int parity, int near, cudaStream_t) {                                     \
+        return enqueue({false, tab, r, n, parity, 0, near});                                                   \
     }
 FAKE_LAUNCHERS(19)
 FAKE_LAUNCHERS(27)
@@ -169,7 +196,7 @@ struct Domains {
     std::vector<std::unique_ptr<lbm_ctx>> own;
     std::vector<lbm_ctx*> ctx;
     std::vector<std::unique_ptr<float>> base;
-    void add(int Q, int nx, int ny, int nz, bool wall_z, float G = -1.0f) {
+    void add(int Q, int nx, int ny, int nz, bool wall_z, float G = -1.0f, bool wall_x = false, bool wall_y = false) {
         own.emplace_back(new lbm_ctx);
         lbm_ctx* c = own.back().get();
         std::memset(&c->kp, 0, sizeof c->kp);
@@ -177,6 +204,8 @@ struct Domains {
         c->kp.nx = nx;
         c->kp.ny = ny;
         c->kp.nz = nz;
+        c->kp.wall_x = wall_x;
+        c->kp.wall_y = wall_y;
         c->kp.wall_z = wall_z;
         c->kp.ncell = c->kp.plane = (long long)nx * ny * nz;
         c->kp.multiphase = 1;
@@ -295,6 +324,38 @@ void odd_calls() {
     }
 }
 
+// Every plane of a tile that holds cells next to a wall has its bit and no other has one, tiles with bits are at most
+// 32 planes high (single planes in launches of the kind that takes no others), and runs that are not marked hold no
+// such cell: for all walls, extents about 32 planes, tile shapes and z-chunks.
+void near_planes() {
+    check_near = true;
+    for (int Q : {19, 27})
+        for (int walls = 0; walls < 8; ++walls) {
+            collided.clear();
+            summed.clear();
+            Domains d;
+            int k = 0;
+            for (int nz : {1, 2, 3, 31, 34, 70}) {
+                d.add(Q, (const int[]){5, 32, 44, 50, 33, 64}[k], (const int[]){9, 1, 4, 6, 13, 8}[k], nz, walls & 4, -1.0f,
+                      walls & 1, walls & 2);
+                ++k;
+            }
+            lbm_batch* b = nullptr;
+            REQUIRE(lbm_batch_create(d.ctx.data(), (int)d.ctx.size(), nullptr, &b) == LBM_OK);
+            long long steps = 0;
+            for (int shape = 0; shape < LBM_BATCH_SHAPES; ++shape)
+                for (int plain : {0, 1, 7, 40, 1 << 30})
+                    for (int solid : {0, 1, 33}) {
+                        REQUIRE(lbm_batch_set_group(b, 0, shape, plain) == LBM_OK);
+                        if (walls) REQUIRE(lbm_batch_set_group(b, 1, shape, solid) == LBM_OK);
+                        REQUIRE(lbm_batch_step(b, 1) == LBM_OK);
+                        d.stepped(++steps);
+                    }
+            lbm_batch_destroy(b);
+            by_base.clear();
+        }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -303,6 +364,7 @@ int main(int argc, char** argv) {
     else if (which == "tune_after_change") retiled_after_change(true);
     else if (which == "set_group_after_change") retiled_after_change(false);
     else if (which == "odd_calls") odd_calls();
+    else if (which == "near_planes") near_planes();
     else return 2;
     std::printf("ok\n");
     return 0;
