@@ -110,6 +110,7 @@ struct lbm_batch {
     std::vector<BatchDom> table;    // member geometry and addresses the groups were built from
     std::vector<Group> groups;
     std::vector<Chain> chains;
+    int sms = 152;                  // of the device
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;     // capture stream
     cudaGraphExec_t exec[2][2] = {};   // [AA phase a call starts from][k]: GRAPH_STEPS[k] steps (nullptr: not recorded)
@@ -238,7 +239,7 @@ std::vector<Column> member_columns(const KParams& k, int tw, int th) {
 // time of the latency / throughput model that choose_zchunk (kernels_impl.cuh) explains; many: four waves
 // of resident blocks, at most ZC_AUTO_MAX planes.
 int auto_zchunk(const lbm_batch* b, const Chain& c, int resident, int tw, int th) {
-    const double cap = 152.0 * resident, ratio = c.Q == 19 ? 6.1 : 5.0;
+    const double sms = b->sms, cap = sms * resident, ratio = c.Q == 19 ? 6.1 : 5.0;
     double planes = 0.0;
     long long cols = 0;
     for (int i : c.members) {
@@ -259,7 +260,7 @@ int auto_zchunk(const lbm_batch* b, const Chain& c, int resident, int tw, int th
             blocks += (double)member_columns(k, tw, th).size() * ((k.nz + zc - 1) / zc);
         }
         const double waves = blocks / cap, B = (zc + 2) * ratio;
-        const double A = blocks / 152.0 * (zc + 1) * (1.0 + 0.15 * (std::ceil(waves) / waves - 1.0));
+        const double A = blocks / sms * (zc + 1) * (1.0 + 0.15 * (std::ceil(waves) / waves - 1.0));
         const double cost = std::max(B, A + 0.35 * B);
         if (cost < best_cost - 1e-9) {
             best_cost = cost;
@@ -283,7 +284,7 @@ lbm_status build_chain(lbm_batch* b, Chain& c) {
     double cells = 0.0;
     for (int i : c.members) cells += (double)b->members[i]->kp.ncell;
     // 2048 cells a run, fewer where that would leave SMs without their eight blocks
-    const uint32_t run_cells = 256u * (uint32_t)std::min(8.0, std::max(1.0, cells / (152.0 * 8.0 * 256.0)));
+    const uint32_t run_cells = 256u * (uint32_t)std::min(8.0, std::max(1.0, cells / (b->sms * 8.0 * 256.0)));
     std::vector<uint8_t> need;      // per plane of one column: needs solid handling
     std::vector<uint8_t> rows;      // per plane and th rows: some column needs solid handling
     for (size_t j0 = 0; j0 < c.members.size(); j0 += lbm::BATCH_LAUNCH_DOMS) {
@@ -375,7 +376,7 @@ lbm_status build_chain(lbm_batch* b, Chain& c) {
         // is faster on D3Q27 in launches of many waves (us a step with walls in z: four 96^3, 3744 tiles, 220.9 / 218.8, ten of
         // 48^3 - 102^3 311.8 / 305.6; but four 72^3, 3060 tiles, 101.6 / 104.0 and four 40^3 21.3 / 22.4; D3Q19 four 96^3
         // 147.4 / 149.1).
-        if (L.near == lbm::NEAR_ENDS && c.Q == 27 && t.size() > 4.5 * 152.0 * sh.minb27) L.near = lbm::NEAR_SOME;
+        if (L.near == lbm::NEAR_ENDS && c.Q == 27 && t.size() > 4.5 * b->sms * sh.minb27) L.near = lbm::NEAR_SOME;
         L.nt = (int)t.size();
         L.nr = (int)runs.size();
         if (L.nt > 0) {
@@ -588,8 +589,11 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int32_t n, void* cuda_stream, 
     lbm_batch* b = new lbm_batch();
     b->members.assign(ctxs, ctxs + n);
     b->stream = (cudaStream_t)cuda_stream;
-    lbm_status s = LBM_OK;
-    s = regroup(b);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+        b->sms = sms;
+    lbm_status s = regroup(b);
     if (s == LBM_OK && cudaStreamSynchronize(b->stream) != cudaSuccess) s = bfail(b, LBM_ERR_CUDA, "batch set-up");
     if (s != LBM_OK) {
         lbm::set_thread_error(b->err.c_str());

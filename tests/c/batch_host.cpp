@@ -29,6 +29,8 @@ namespace {
 std::map<const char*, size_t> live;   // allocations
 int allocs_left = -1;                 // cudaMalloc calls that still succeed (-1: all)
 int instantiated = 0;
+int device_sms = 152;
+int last_runs = 0;                    // of the last density pass
 
 struct Pass {
     bool collide;
@@ -97,6 +99,7 @@ void check(const Pass& p) {
             REQUIRE(r.end <= n && collided[d.base] % n == 0);
             REQUIRE(p.parity == (int)(collided[d.base] / n % 2));
             summed[d.base] += r.end - r.begin;
+            last_runs = p.n;
             if (check_near) check_run(p, r, d);
         }
     }
@@ -144,7 +147,7 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cu
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaErrorMemoryAllocation ? "out of memory" : "error"; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
-cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = device_sms, cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { return *e = handle<cudaEvent_t>(), cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { return delete (char*)e, cudaSuccess; }
@@ -356,6 +359,24 @@ void near_planes() {
         }
 }
 
+// Work is cut for the SMs that the device has: 2432 x 256 cells in runs for eight blocks each.
+void sm_count() {
+    for (int sms : {152, 76, 304}) {
+        device_sms = sms;
+        collided.clear();
+        summed.clear();
+        Domains d;
+        d.add(19, 128, 64, 76, false);
+        lbm_batch* b = nullptr;
+        REQUIRE(lbm_batch_create(d.ctx.data(), 1, nullptr, &b) == LBM_OK);
+        REQUIRE(lbm_batch_step(b, 1) == LBM_OK);
+        d.stepped(1);
+        REQUIRE(last_runs == (sms == 76 ? 608 : sms == 152 ? 1216 : 2432));
+        lbm_batch_destroy(b);
+        by_base.clear();
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -365,6 +386,7 @@ int main(int argc, char** argv) {
     else if (which == "set_group_after_change") retiled_after_change(false);
     else if (which == "odd_calls") odd_calls();
     else if (which == "near_planes") near_planes();
+    else if (which == "sm_count") sm_count();
     else return 2;
     std::printf("ok\n");
     return 0;

@@ -31,7 +31,7 @@ def program(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["failed_rebuild", "tune_after_change", "set_group_after_change", "odd_calls",
-                                      "near_planes"])
+                                      "near_planes", "sm_count"])
 def test_batch_host(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and r.stdout == "ok\n", (r.returncode, r.stdout, r.stderr)
