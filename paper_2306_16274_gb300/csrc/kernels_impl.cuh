@@ -149,8 +149,10 @@ __device__ __forceinline__ int swept_block(int down) {
 }
 
 // MIXED: solid handling in the planes that the column's SolidPlanes name
+// FP16 store, one slot per cell, no solids: for 16 blocks per SM (32 registers; the compiler's own choice is 40 on the even
+// phase): us a pass, compiler's choice / this, D3Q19 256^3 218.2 / 211.9, D3Q27 289.1 / 277.9.
 template <int PARITY, bool MIXED, bool F16>
-__global__ void __launch_bounds__(PSI_BX * PSI_BY) psi_kernel(KParams kp, float* __restrict__ psi,
+__global__ void __launch_bounds__(PSI_BX * PSI_BY, F16 && !MIXED ? 16 : 0) psi_kernel(KParams kp, float* __restrict__ psi,
                                                             const uint32_t* __restrict__ nbmask, unsigned* status,
                                                             const float* __restrict__ rsrc,
                                                             float* __restrict__ rdst,
