@@ -798,9 +798,11 @@ __device__ __forceinline__ void psi_pairs(const KParams& kp, float* __restrict__
 // 879 against 865; 10 blocks 638 and 975.
 // MIXED: solid handling in the planes that SolidPlanes names (no mask in this layout: at walls in y and z).  With it
 // in all planes of a domain with walls / in those alone, us a step: D3Q19 400 x 400 x 200 1448 / 1328, D3Q27
-// 200 x 200 x 100 319 / 289; one slot per cell (psi_kernel) 201 x 200 x 100 219 / 199.
+// 200 x 200 x 100 319 / 289; one slot per cell (psi_kernel) 201 x 200 x 100 219 / 199.  MIXED on D3Q27 spills at 64 registers
+// (76 bytes), so 6 blocks: with walls in y, 8 / 6 blocks, 32^3 23.4 / 20.1, 127^3 177.8 / 169.3, z walls 200 x 200 x 100
+// 290 / 281.
 template <int PARITY, bool MIXED>
-__global__ void __launch_bounds__(PSI_BX * PSI_BY, 8) psi_pair_kernel(const KParams kp, float* __restrict__ psi,
+__global__ void __launch_bounds__(PSI_BX * PSI_BY, MIXED && LBM_Q == 27 ? 6 : 8) psi_pair_kernel(const KParams kp, float* __restrict__ psi,
                                                                     unsigned* status, const float* __restrict__ rsrc,
                                                                     float* __restrict__ rdst) {
     const int z = swept_block(kp.down);
@@ -922,16 +924,21 @@ __device__ __forceinline__ void collide_pair_tile(const KParams& kp, const float
     }
 }
 
-template <int PARITY, bool MULTIPHASE>
+template <int PARITY, bool MULTIPHASE, bool ROOMY = false>
 __device__ __noinline__ void collide_pair_tile_near(const KParams& kp, const float* psi, unsigned* status, int z0, int zend,
                                                     const float* rsrc, const float* rown, float (*ring)[2][PR_RP],
                                                     float (*rring)[2][PR_RP]) {
     collide_pair_tile<PARITY, true, MULTIPHASE>(kp, psi, status, z0, zend, rsrc, rown, ring, rring);
 }
 
-// NEAR as in collide_kernel (no mask in this layout: only cells at walls in y and z have solid neighbours)
-template <int PARITY, int NEAR, bool MULTIPHASE>
-__global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const __grid_constant__ KParams kp,
+// NEAR as in collide_kernel (no mask in this layout: only cells at walls in y and z have solid neighbours).  ROOMY: fewer
+// blocks per SM, so that the function for columns at walls in y spills less (D3Q19 396 -> 28, D3Q27 476 -> 172 bytes at most), for
+// domains whose single planes of columns all fit the SMs at once and so wait for those columns: us a step with walls
+// in y, without / with it, D3Q19 32^3 15.3 / 13.7, 48^3 19.5 / 15.2 (64^3, where they do not fit, 20.3 / 20.9); D3Q27 32^3 20.0 /
+// 19.3, 40^3 22.6 / 19.6 (48^3 21.3 / 23.4).
+constexpr int PR_MINB_ROOMY = LBM_Q == 19 ? 4 : 3;
+template <int PARITY, int NEAR, bool MULTIPHASE, bool ROOMY = false>
+__global__ void __launch_bounds__(PR_NT, ROOMY ? PR_MINB_ROOMY : PR_MINB) collide_pair_kernel(const __grid_constant__ KParams kp,
                                                                      const float* __restrict__ psi,
                                                                      unsigned* status, int zchunk,
                                                                      const float* __restrict__ rsrc,
@@ -958,7 +965,7 @@ __global__ void __launch_bounds__(PR_NT, PR_MINB) collide_pair_kernel(const __gr
         SolidPlanes sp(KGeom{kp}, nullptr, 0, blockIdx.y * PR_BY, 0, PR_BY, 0, 0);
         for_plane_runs(sp, z0, min(z0 + zchunk, kp.nz), [&](bool solids, int za, int zb) {
             if (solids)
-                collide_pair_tile_near<PARITY, MULTIPHASE>(kp, psi, status, za, zb, rsrc, rown, ring, rring);
+                collide_pair_tile_near<PARITY, MULTIPHASE, ROOMY>(kp, psi, status, za, zb, rsrc, rown, ring, rring);
             else
                 collide_pair_tile<PARITY, false, MULTIPHASE>(kp, psi, status, za, zb, rsrc, rown, ring, rring);
         });
@@ -1704,14 +1711,14 @@ cudaError_t launch_collide_store(dim3 g, dim3 b, cudaStream_t st, const KParams&
                          : launch_collide_variant<1, NEAR, false, F16>(g, b, st, kp, B, zc);
 }
 
-template <int NEAR>
+template <int NEAR, bool ROOMY = false>
 cudaError_t launch_collide_pairs(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, const Bufs& B, int zc, int parity) {
     const float *r0 = B.rsrc, *r1 = B.rnew;
     if (parity == 0)
-        return kp.multiphase ? launch_dep(collide_pair_kernel<0, NEAR, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1)
-                             : launch_dep(collide_pair_kernel<0, NEAR, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
-    return kp.multiphase ? launch_dep(collide_pair_kernel<1, NEAR, true>, g, b, st, kp, B.psi, B.status, zc, r0, r1)
-                         : launch_dep(collide_pair_kernel<1, NEAR, false>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+        return kp.multiphase ? launch_dep(collide_pair_kernel<0, NEAR, true, ROOMY>, g, b, st, kp, B.psi, B.status, zc, r0, r1)
+                             : launch_dep(collide_pair_kernel<0, NEAR, false, ROOMY>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
+    return kp.multiphase ? launch_dep(collide_pair_kernel<1, NEAR, true, ROOMY>, g, b, st, kp, B.psi, B.status, zc, r0, r1)
+                         : launch_dep(collide_pair_kernel<1, NEAR, false, ROOMY>, g, b, st, kp, B.psi, B.status, zc, r0, r1);
 }
 
 template <bool F16>
@@ -1785,6 +1792,17 @@ cudaError_t LBM_CAT(launch_psi_q, LBM_Q)(const KParams& kp, int parity, int soli
                  : launch_psi_store<false>(g, b, st, kp, parity, solids, B);
 }
 
+static int device_sms() {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
+                                                      cudaSuccess || n <= 0)
+            n = 152;
+        return n;
+    }();
+    return sms;
+}
+
 // z-planes per block of the z-marching kernels.  Blocks of equal size run in waves of
 // (SMs x resident blocks); a last wave that is mostly empty leaves SMs idle, and every chunk
 // costs about h planes' worth of extra time at its start (the psi planes below and at its first
@@ -1802,13 +1820,7 @@ cudaError_t LBM_CAT(launch_psi_q, LBM_Q)(const KParams& kp, int parity, int soli
 static int choose_zchunk(const KParams& kp, double h, int nz, int by, int minb) {
     if (kp.zchunk > 0) return kp.zchunk < nz ? kp.zchunk : nz;
     if (nz <= 1) return 1;
-    static const int sms = [] {
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
-                                                      cudaSuccess || n <= 0)
-            n = 152;
-        return n;
-    }();
+    const int sms = device_sms();
     thread_local long long key[4] = {-1, -1, -1, -1};
     thread_local int cached = 1;
     const long long k[4] = {kp.nx, kp.ny, nz, (long long)(h * 1024.0) + 4096LL * (by + 64LL * minb)};
@@ -1852,6 +1864,8 @@ cudaError_t LBM_CAT(launch_collide_q, LBM_Q)(const KParams& kp, int parity, int 
     static_assert(PR_BX == ZM_BX && PR_BY == ZM_BY, "one grid for both");
     const dim3 g((kw.nx + ZM_BX - 1) / ZM_BX, (kp.ny + ZM_BY - 1) / ZM_BY, (planes + zc - 1) / zc + (ends ? 2 : 0)),
         b(ZM_BX, ZM_BY);
+    if (B.paired && near == NEAR_SOME && (double)g.x * g.y * kp.nz <= (double)device_sms() * PR_MINB_ROOMY)
+        return launch_collide_pairs<NEAR_SOME, true>(g, b, st, kp, B, zc, parity);
     if (B.paired)
         return near == NEAR_NONE   ? launch_collide_pairs<NEAR_NONE>(g, b, st, kp, B, zc, parity)
                : near == NEAR_ENDS ? launch_collide_pairs<NEAR_ENDS>(g, b, st, kp, B, zc, parity)
