@@ -515,8 +515,11 @@ __device__ __noinline__ void collide_tile_near(const KParams& kp, const float* p
 // as two launches a pass over tile lists, replayed from a graph / as one kernel: D3Q19 127 x 127 x 106 92.5 /
 // 77.8, 256^3 746 / 672, D3Q27 127 x 127 x 106 130.9 / 107.1.  (As a march cut into runs with and without solids,
 // each through its own copy of the tile: 87.9, 709 and 127.6 us; registers spill in the plain copy.)
-template <int PARITY, int NEAR, bool MULTIPHASE, bool F16>
-__global__ void __launch_bounds__(ZmTile::NT, ZM_MINB) collide_kernel(const __grid_constant__ KParams kp,
+// ROOMY: one block per SM fewer; single-phase FP32 tiles that switch from plane to plane spill otherwise (142 bytes on the odd phase of
+// D3Q19): us a step with walls in x / a cylinder, without and with it, D3Q19 48^3 6.6 / 5.9 and 6.5 / 6.1, 80^3 20.5 / 17.1 and 18.9 /
+// 15.6, 127^3 61.0 / 53.4 and 60.0 / 52.4; D3Q27 48^3 8.9 / 7.3 and 8.4 / 6.9, 127^3 80.2 / 75.1 and 78.6 / 73.5.
+template <int PARITY, int NEAR, bool MULTIPHASE, bool F16, bool ROOMY = false>
+__global__ void __launch_bounds__(ZmTile::NT, ZM_MINB - ROOMY) collide_kernel(const __grid_constant__ KParams kp,
                                                                 const float* __restrict__ psi,
                                                                 const uint32_t* __restrict__ nbmask,
                                                                 unsigned* status, int zchunk,
@@ -1688,18 +1691,19 @@ cudaError_t launch_dep(void (*kernel)(KA...), dim3 g, dim3 b, cudaStream_t st, c
 #ifndef LBM_ZM_CARVEOUT
 #define LBM_ZM_CARVEOUT -1
 #endif
-template <int PARITY, int NEAR, bool MULTIPHASE, bool F16>
+template <int PARITY, int NEAR, bool MULTIPHASE, bool F16, bool ROOMY = false>
 cudaError_t launch_collide_variant(dim3 g, dim3 b, cudaStream_t st, const KParams& kp, const Bufs& B, int zc) {
     if (LBM_ZM_CARVEOUT >= 0) {
         static bool configured = false;
         if (!configured) {
-            cudaError_t e = cudaFuncSetAttribute(collide_kernel<PARITY, NEAR, MULTIPHASE, F16>,
+            cudaError_t e = cudaFuncSetAttribute(collide_kernel<PARITY, NEAR, MULTIPHASE, F16, ROOMY>,
                                                  cudaFuncAttributePreferredSharedMemoryCarveout, LBM_ZM_CARVEOUT);
             if (e != cudaSuccess) return e;
             configured = true;
         }
     }
-    return launch_dep(collide_kernel<PARITY, NEAR, MULTIPHASE, F16>, g, b, st, kp, B.psi, B.nbmask, B.status, zc, B.rsrc, B.rnew, B.zmask);
+    return launch_dep(collide_kernel<PARITY, NEAR, MULTIPHASE, F16, ROOMY>, g, b, st, kp, B.psi, B.nbmask, B.status, zc, B.rsrc,
+                      B.rnew, B.zmask);
 }
 
 template <int NEAR, bool F16>
@@ -1860,7 +1864,14 @@ cudaError_t LBM_CAT(launch_collide_q, LBM_Q)(const KParams& kp, int parity, int 
     const int planes = kp.nz - (ends ? 2 : 0);
     KParams kw = kp;   // pairs: tiles of 32 words, so the z-chunk choice counts columns of hx words
     if (B.paired) kw.nx = kp.hx;
-    const int zc = B.paired ? choose_zchunk(kw, 1.0, planes, PR_BY, PR_MINB) : choose_zchunk(kp, 1.0, planes, ZM_BY, ZM_MINB);
+    int zc = B.paired ? choose_zchunk(kw, 1.0, planes, PR_BY, PR_MINB) : choose_zchunk(kp, 1.0, planes, ZM_BY, ZM_MINB);
+    bool roomy = near == NEAR_SOME && !kp.multiphase && !B.f16;
+    if (roomy && kp.zchunk == 0) {
+        // not where marches of two planes just fit the SMs with the one block more (64^3 D3Q19: 9.6 against 10.5)
+        const long long blocks = (long long)((kp.nx + ZM_BX - 1) / ZM_BX) * ((kp.ny + ZM_BY - 1) / ZM_BY) * ((planes + zc - 1) / zc);
+        if (zc <= 2 && blocks <= (long long)device_sms() * ZM_MINB && blocks > (long long)device_sms() * (ZM_MINB - 1)) roomy = false;
+        else zc = choose_zchunk(kp, 1.0, planes, ZM_BY, ZM_MINB - 1);
+    }
     static_assert(PR_BX == ZM_BX && PR_BY == ZM_BY, "one grid for both");
     const dim3 g((kw.nx + ZM_BX - 1) / ZM_BX, (kp.ny + ZM_BY - 1) / ZM_BY, (planes + zc - 1) / zc + (ends ? 2 : 0)),
         b(ZM_BX, ZM_BY);
@@ -1874,6 +1885,9 @@ cudaError_t LBM_CAT(launch_collide_q, LBM_Q)(const KParams& kp, int parity, int 
         return near == NEAR_NONE   ? launch_collide_store<NEAR_NONE, true>(g, b, st, kp, B, zc, parity)
                : near == NEAR_ENDS ? launch_collide_store<NEAR_ENDS, true>(g, b, st, kp, B, zc, parity)
                                    : launch_collide_store<NEAR_SOME, true>(g, b, st, kp, B, zc, parity);
+    if (roomy)
+        return parity == 0 ? launch_collide_variant<0, NEAR_SOME, false, false, true>(g, b, st, kp, B, zc)
+                           : launch_collide_variant<1, NEAR_SOME, false, false, true>(g, b, st, kp, B, zc);
     return near == NEAR_NONE   ? launch_collide_store<NEAR_NONE, false>(g, b, st, kp, B, zc, parity)
            : near == NEAR_ENDS ? launch_collide_store<NEAR_ENDS, false>(g, b, st, kp, B, zc, parity)
                                : launch_collide_store<NEAR_SOME, false>(g, b, st, kp, B, zc, parity);

@@ -30,3 +30,27 @@ def test_pairs_at_side_walls(Q, shape, bc):
         single.step(n)
         assert np.array_equal(pairs.populations(device=False), single.populations(device=False)), n
         assert np.array_equal(pairs.psi(device=False), single.psi(device=False)), n
+
+
+@pytest.mark.parametrize("Q", [19, 27])
+@pytest.mark.parametrize("shape", [(64, 64, 64), (64, 64, 60), (20, 7, 1), (33, 130, 40)], ids=str)
+@pytest.mark.parametrize("bc,points,zchunk", [((1, 0, 0), 0, 0), ((0, 1, 1), 0, 0), ((0, 0, 1), 5, 0), ((0, 0, 0), 5, 3),
+                                              ((0, 0, 1), 0, 0)], ids=str)
+def test_single_phase_walls_and_solids(Q, shape, bc, points, zchunk):
+    from paper_2306_16274_gb300 import Batch
+    nx, ny, nz = shape
+    rho, u = W.perturbed(shape, seed=5)
+    mask = None
+    if points:
+        rng = np.random.default_rng(nx + nz)
+        mask = np.zeros((nz, ny, nx), dtype=np.uint8)
+        for _ in range(points):
+            mask[rng.integers(nz), rng.integers(ny), rng.integers(nx)] = 1
+    d = dict(lattice=Q, shape=shape, bc=bc, zchunk=zchunk)
+    alone, member = U.run_gpu(d, rho, u, mask), U.run_gpu(d, rho, u, mask)
+    b = Batch([member])
+    for n in (1, 1, 6):
+        alone.step(n)
+        b.step(n)
+        assert np.array_equal(alone.populations(device=False), member.populations(device=False)), n
+    b.close()
