@@ -165,9 +165,9 @@ lbm_status lbm_init_fields(lbm_ctx* ctx, const float* rho, const float* u, const
                            int ptrs_on_device);
 
 /* Enqueues n >= 0 time steps on the context's stream and returns without
- * waiting.  Returns a sticky error recorded by an earlier lbm_sync.  A domain
- * with walls or solids is stepped through the tile path of the batches below
- * (same results, solid-free tiles skip the solid tests). */
+ * waiting.  Returns a sticky error recorded by an earlier lbm_sync.  In a domain
+ * with walls or solids only the planes, column by column, that hold cells next to
+ * them take the code with solid tests. */
 lbm_status lbm_step(lbm_ctx* ctx, int32_t n);
 
 /* Waits for the context's stream and reads the device status word:
@@ -245,9 +245,9 @@ void lbm_destroy(lbm_ctx* ctx);
 /* ---------------------------------------------------------------- batches
  * Many independent domains advanced together (the paper's method applied to a set
  * of jobs; the paper itself runs one domain at a time).  Every member is cut into
- * tiles (32 x 4 columns by default, see LBM_BATCH_SHAPES) and runs of z planes; a
- * tile whose cells have no solid
- * neighbour (mask or wall) goes to a group without solid handling.  Groups are
+ * tiles (32 x 4 columns by default, see LBM_BATCH_SHAPES, and chunks of z planes); a
+ * tile whose cells have no solid neighbour (mask or wall) belongs to a group without
+ * solid handling, the others tell plane by plane where they need it.  Groups are
  * keyed by (lattice, solid handling, physical parameters); the groups of one lattice
  * and physics are stepped together: each time step costs, per 64 of their members, one
  * collide-stream launch and one density/psi launch whose blocks are tiles of all those
@@ -275,7 +275,8 @@ void lbm_destroy(lbm_ctx* ctx);
  *   the fastest shape, each candidate z-chunk (automatic, 1, 4, 8, 16, 32 planes
  *   per block, or a whole column per block).  A group and the group of the same lattice and physics
  *   with the other solid handling share members and launches, so they are timed together and
- *   take one shape.  Keeps the fastest per group and writes its z-chunk to
+ *   take one shape and one z-chunk (lbm_batch_set_group can give them different z-chunks).
+ *   Keeps the fastest and writes the z-chunk of group g to
  *   zchunk_out[g] for g < max_groups (0 = automatic, 2^30 = whole columns;
  *   lbm_batch_group reads the shape).  The members advance by 12 x (trial_steps + 1) steps.
  * lbm_batch_info: number of groups, tiles of all launches of one pass, graph mode
@@ -284,7 +285,8 @@ void lbm_destroy(lbm_ctx* ctx);
  * lbm_batch_group: lattice (19 | 27), solid handling (0 | 1), tile shape and
  *   z-chunk of group `group` in [0, ngroups); NULL outputs are skipped.
  * lbm_batch_set_group: sets a group's tile shape (0 .. LBM_BATCH_SHAPES - 1) and
- *   z-chunk (0 = automatic) and re-tiles it; the group of the same lattice and
+ *   z-chunk (0 = automatic) and re-tiles it (a tile with solid handling is at most 32
+ *   planes high whatever the z-chunk); the group of the same lattice and
  *   physics with the other solid handling takes the same shape.  Results do not
  *   depend on either.
  *   LBM_ERR_ARG for an unknown group, shape or a negative z-chunk.

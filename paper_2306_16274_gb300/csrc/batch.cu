@@ -7,8 +7,8 @@
 // (geometry and buffer addresses) are passed by value in the kernel parameters, so a block reads them from the
 // constant bank as the single-domain kernel does.  The per-cell arithmetic is the single-domain code, so a
 // member's result is bitwise the same as stepping it alone.  The chains run side by side on streams of their
-// own, joined once a call; runs of steps are replayed from CUDA graphs of 2 and 16 steps, within which the
-// kernels of a chain overlap at their ends as lbm_step's do.
+// own; runs of steps are replayed from CUDA graphs of 2 and 16 steps, within which the kernels of a chain
+// overlap at their ends as lbm_step's do, and at whose ends the chains are joined.
 // us a step, one launch a group and pass with all groups joined after every pass, in a device-side loop / this:
 // 4 x 32^3 D3Q19 17.2 / 8.8; 40^3 droplets and impacts on both lattices 34.0 / 19.4; 8 x 64^3 93.9 / 85.1; ten mixed
 // jobs of 48^3 - 109^3 318 / 290; 24 mixed jobs of 48^3 - 160^3 1665 / 1636.  (Advancing members in bins that fit the L2
@@ -505,7 +505,7 @@ lbm_status refresh(lbm_batch* b) {
 
 // `steps` steps of every member from AA phase `parity` (psi of the current state valid).  Within a chain a step
 // needs the one before it (psi reads populations that neighbouring tiles wrote, collide the psi halo); the chains
-// have nothing in common, so each runs all its steps on a stream of its own, joined at the end.
+// have nothing in common, so each runs all these steps on a stream of its own, joined at the end.
 cudaError_t step_all(lbm_batch* b, int parity, int steps, cudaStream_t st) {
     auto steps_of = [&](const Chain& c, cudaStream_t s) {
         cudaError_t e = cudaSuccess;

@@ -253,8 +253,10 @@ __device__ __forceinline__ void denorm(float (&p)[Q], uint32_t bits, const RS& r
 }
 
 // Density of a cell of a domain with walls or solids from its slot values, every rounding written out: cells
-// with and without solid neighbours take different code, and the density must not depend on which.  (Each
-// product is rounded before it is added, but the last.)
+// with and without solid neighbours take different code, and the density must not depend on which.  Each
+// product is rounded before it is added, but the last: as the compiler had fused the sum before it was written
+// out, kept so that results stayed the same bits.  Domains without walls have one code, whose fusing is left to the
+// compiler (denorm and a sum), and may round otherwise.
 template <int Q, bool SOLIDS, class RS>
 __device__ __forceinline__ float denorm_sum(const float (&p)[Q], uint32_t bits, const RS& rs) {
     const float self = rs.at(0, 0, 0);
