@@ -282,7 +282,7 @@ def batch_jobs(n_jobs=64, seed=2306):
 
 def run_batched(steps, n_jobs=64):
     """The same jobs advanced one at a time (each job's `steps` steps through the plain single-domain
-    kernels, jobs back to back) and together (one tuned batch, one graph launch)."""
+    kernels, jobs back to back) and together (one tuned batch, replayed graphs)."""
     import torch
 
     from paper_2306_16274_gb300 import Batch, Params, Simulation
